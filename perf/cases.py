@@ -379,3 +379,83 @@ def tolerance(case):
     if case["kind"] in ("forward", "decode_lfu"):
         return {"rel": 1e-2, "max": 0.04}
     return {"rel": 1.3e-2, "max": 0.9}
+
+
+# ---- the same outputs in 64 bits, in plain torch ------------------------------------------------------
+def _pad_rows(t, rows):
+    out = torch.zeros((rows,) + tuple(t.shape[1:]), dtype=t.dtype, device=t.device)
+    out[:t.shape[0]] = t
+    return out
+
+
+def _exact_layer(x, ids, dy, W_gate, W_down, E, W_up=None):
+    """The layer's formulas in fp64 (dy None: the forward alone); table-gradient rows of the distinct
+    ids in ascending order."""
+    ids = ids.long()
+    x, Wg, Wd = x.double(), W_gate.double(), W_down.double()
+    u = E[ids].double()
+    if W_up is not None:
+        u = u + x @ W_up.double().T
+    g = x @ Wg.T
+    s = torch.sigmoid(g)
+    h = g * s * u
+    o = {"y": h @ Wd.T}
+    if dy is None:
+        return o
+    dy = dy.double()
+    o.update(G=g, H=h, U=u)
+    dh = dy @ Wd
+    o["dW_down"] = dy.T @ h
+    du = dh * (g * s)
+    dg = dh * u * (s * (1 + g * (1 - s)))
+    o["dx"] = dg @ Wg
+    o["dW_gate"] = dg.T @ x
+    if W_up is not None:
+        o["dx"] = o["dx"] + du @ W_up.double()
+        o["dW_up"] = du.T @ x
+    unique, inverse = torch.unique(ids, return_inverse=True)
+    o["dE_rows"] = torch.zeros(unique.numel(), E.shape[1], dtype=torch.float64, device=u.device).index_add_(0, inverse, du)
+    return o
+
+
+def _exact_state(st, more=(), W_up=None):
+    e = _exact_layer(st.x, st.ids, st.dy, st.W_gate, st.W_down, st.E, W_up)
+    e["dE_rows"] = _pad_rows(e["dE_rows"], st.bufs["dE_rows"].shape[0])
+    out = {k: e[k] for k in ("y",) + tuple(more) + GRADS}
+    out.update({k: None for k in INDEX})         # whole numbers: either side has the one right value
+    return out
+
+
+def exact(case, seed):
+    """What `run` returns for these inputs, in 64 bits (None for the index arrays and counters)."""
+    s = prepare(case, seed)
+    kind = case["kind"]
+    if kind == "forward":
+        st = s["st"]
+        return _exact_layer(st.x, st.ids, None, st.W_gate, st.W_down, st.E)["y"]
+    if kind == "train":
+        return _exact_state(s["st"], ("G", "H"))
+    if kind == "micro":
+        parts = [_exact_state(st) for st in s["parts"]]
+        for k in ("dW_gate", "dW_down"):         # both micro-batches add to the same buffers
+            parts[0][k] = parts[1][k] = parts[0][k] + parts[1][k]
+        return parts
+    if kind == "dagger":
+        return _exact_state(s["st"], ("G", "H", "U", "dW_up"), s["W_up"])
+    if kind == "decode_lfu":
+        st, table = s["st"], s["table"].cuda()
+        y = [_exact_layer(x, ids, None, st.W_gate, st.W_down, table)["y"] for ids, x in zip(s["ids"], s["x"])]
+        return {"y": y, "freq": None, "hits": None, "rows": None}
+    if kind == "host_stack":
+        stack = s["stack"]
+        layers, host = [], []
+        for i in range(case["layers"]):
+            e = _exact_layer(s["x"][i], s["ids"][i], s["dy"][i], stack.W_gate, stack.W_down, stack.tables[i].cuda())
+            layers.append({k: e[k] for k in ("y", "dx", "dW_gate", "dW_down")})
+            host.append({"host_rows": _pad_rows(e["dE_rows"], stack.R), "host_ids": None, "host_n": None})
+        return {"layers": layers, "host": host}
+    h = {k: s["host"][k].cuda() for k in ("x", "ids", "dy")}
+    e = _exact_layer(h["x"], h["ids"], h["dy"], s["W_gate"], s["W_down"], s["E"])
+    out = {k: e[k] for k in ("y", "dx", "dW_gate", "dW_down")}
+    out.update(dE_rows=_pad_rows(e["dE_rows"], s["dE_rows"].shape[0]), n=None, unique_ids=None)
+    return out
