@@ -28,7 +28,8 @@
  *     workspace's status word and read back with stem_query_status().  A bad id is
  *     clamped into range so no access leaves the table.  Nothing traps, prints from the
  *     device or throws; there is no CPU fallback.
- *   - dtype 0: fp32 storage and fp32 FMA arithmetic.  dtype 1: bf16 storage, bf16
+ *   - dtype 0: fp32 storage, fp32 products and sums (on the tensor cores, three bf16 parts
+ *     per operand).  dtype 1: bf16 storage, bf16
  *     tensor-core products accumulated in fp32, elementwise math in fp32, results
  *     rounded to bf16 (round to nearest even) when stored.
  *   - Shape limits: T <= 2^22; d_model and d_ff multiples of 8 (bf16) or 4 (fp32);
@@ -59,7 +60,7 @@ extern "C" {
 #define STEM_DTYPE_FP32 0
 #define STEM_DTYPE_BF16 1
 
-#define STEM_FLAG_SIMT 1 /* run the bf16 contractions on the plain-FMA kernels (debug aid) */
+#define STEM_FLAG_SIMT 1 /* run the contractions on the plain-FMA kernels (debug aid) */
 #define STEM_FLAG_SINGLE_CTA 2 /* tensor-core contractions on single CTAs instead of CTA pairs (debug aid) */
 /* Backward adds the weight gradients (dW_gate, dW_down, and dW_up of the dagger variant) to what
  * the caller's buffers hold instead of overwriting them: gradient accumulation over

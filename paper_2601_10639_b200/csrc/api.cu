@@ -2,6 +2,7 @@
 #include <atomic>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <mutex>
 #include <vector>
 
@@ -116,6 +117,7 @@ struct WsLayout {
   size_t dedup_off, dedup_bytes;
   size_t h_off, h_bytes;     // forward: H when the caller keeps none
   size_t du_off, dg_off, tf_bytes, part_off, part_bytes, sk_off, sk_bytes;
+  size_t x3_off, dy3_off, wg3_off, wd3_off, h3_off, dg3_off;   // fp32: the operands' bf16 parts
   size_t total;
 };
 
@@ -137,6 +139,16 @@ WsLayout ws_layout(const stem_shape_t* s) {
   size_t m = w.dedup_off + w.dedup_bytes;
   if (w.h_off + w.h_bytes > m) m = w.h_off + w.h_bytes;
   if (w.sk_off + w.sk_bytes > m) m = w.sk_off + w.sk_bytes;
+  if (s->dtype == STEM_DTYPE_FP32) {
+    m = align_up(m, 1024);
+    const size_t td = parts_bytes(s->T, s->d_model), fd = parts_bytes(s->d_ff, s->d_model), df = parts_bytes(s->d_model, s->d_ff),
+                 tf3 = parts_bytes(s->T, s->d_ff);
+    w.x3_off = m; w.dy3_off = w.x3_off + td; w.wg3_off = w.dy3_off + td;
+    w.wd3_off = w.wg3_off + fd;
+    // (the dagger variant keeps W_up's parts where W_down's were or will be: either orientation fits)
+    w.h3_off = w.wd3_off + (df > fd ? df : fd); w.dg3_off = w.h3_off + tf3;
+    m = w.dg3_off + tf3;
+  }
   w.total = align_up(m, 256);
   return w;
 }
@@ -145,6 +157,40 @@ int32_t* status_of(void* ws) { return static_cast<int32_t*>(ws); }
 
 bool use_tc(const stem_shape_t* s) {
   return s->dtype == STEM_DTYPE_BF16 && !(s->flags & STEM_FLAG_SIMT);
+}
+
+// fp32 on the tensor cores (three bf16 parts per operand)
+bool use_split(const stem_shape_t* s) {
+  return s->dtype == STEM_DTYPE_FP32 && !(s->flags & STEM_FLAG_SIMT) && is_sm100();
+}
+
+// An fp32 operand and where its parts lie in the workspace.
+struct Operand { const float* m; Parts p; };
+Operand operand(const void* ws, size_t off, const void* m, int rows, int cols) {
+  Operand o{static_cast<const float*>(m), Parts{}};
+  o.p.base = const_cast<char*>(static_cast<const char*>(ws)) + off;
+  o.p.rows = rows; o.p.cols = cols; o.p.pitch = (cols + 7) / 8 * 8;
+  return o;
+}
+cudaError_t split3(std::initializer_list<Operand> ops, cudaStream_t st) {
+  SplitJob jobs[kMaxSplitJobs];
+  int n = 0;
+  for (const Operand& o : ops) {
+    if (n == kMaxSplitJobs) return cudaErrorInvalidValue;
+    jobs[n++] = {o.m, o.p};
+  }
+  return launch_split3(jobs, n, st);
+}
+SplitProduct split_product(const Operand& a, const Operand& b, void* out, int M, int N) {
+  SplitProduct p;
+  p.A = a.m; p.B = b.m; p.A3 = a.p; p.B3 = b.p;
+  p.out = static_cast<float*>(out);
+  p.M = M; p.N = N;
+  return p;
+}
+cudaError_t split_gemm(int M, int N, int K, const Operand& a, bool a_mn, const Operand& b, bool b_mn, EpiKind kind,
+                       const EpiParams& ep, cudaStream_t st) {
+  return launch_split_gemm(split_product(a, b, ep.out, M, N), SplitProduct{}, K, a_mn, b_mn, kind, ep, st);
 }
 
 cudaError_t gemm(const stem_shape_t* s, int M, int N, int K, const void* A, bool a_mn, const void* B,
@@ -244,6 +290,26 @@ int stem_ffn_forward(const stem_shape_t* shape, const void* x, const int32_t* id
   EpiParams gate;
   gate.ids = ids; gate.E = E; gate.V = shape->V; gate.H = H; gate.G = G_save; gate.status = status_of(ws);
   cudaError_t e;
+  if (use_split(shape)) {
+    const Operand x3 = operand(ws, w.x3_off, x, T, d), wg3 = operand(ws, w.wg3_off, W_gate, F, d),
+                  wd3 = operand(ws, w.wd3_off, W_down, d, F), h3 = operand(ws, w.h3_off, H, T, F);
+    {
+      ProfScope prof("split_operands", st);
+      e = split3({x3, wg3, wd3}, st);
+    }
+    if (e != cudaSuccess) return cuda_fail(e);
+    gate.H3 = h3.p;
+    {
+      ProfScope prof("gate_gemm", st);
+      e = split_gemm(T, F, d, x3, false, wg3, false, kEpiGate, gate, st);
+    }
+    if (e != cudaSuccess) return cuda_fail(e);
+    EpiParams down;
+    down.out = y; down.status = status_of(ws);
+    ProfScope prof("down_gemm", st);
+    e = split_gemm(T, d, F, h3, false, wd3, false, kEpiStore, down, st);
+    return e == cudaSuccess ? STEM_OK : cuda_fail(e);
+  }
   {
     ProfScope prof("gate_gemm", st);
     e = gemm(shape, T, F, d, x, false, W_gate, false, kEpiGate, gate, st);   // G = x W_gate^T, fused lookup
@@ -291,7 +357,22 @@ int stem_ffn_backward(const stem_shape_t* shape, const void* dy, const void* x, 
   EpiParams dh;
   dh.ids = ids; dh.E = E; dh.V = shape->V; dh.H = dU; dh.G = dG; dh.Gin = G_save; dh.status = status_of(ws);
   cudaError_t e;
-  {
+  const bool split = use_split(shape);
+  const Operand dy3 = operand(ws, w.dy3_off, dy, T, d), x3 = operand(ws, w.x3_off, x, T, d),
+                wg3 = operand(ws, w.wg3_off, W_gate, F, d), wd3 = operand(ws, w.wd3_off, W_down, d, F),
+                h3 = operand(ws, w.h3_off, H_save, T, F), dg3 = operand(ws, w.dg3_off, dG, T, F);
+  if (split) {
+    {
+      ProfScope prof("split_operands", st);
+      // the operands of the outputs that are asked for; dG's parts come from the dH epilogue
+      Operand none{};
+      e = split3({dy3, wd3, dW_gate ? x3 : none, dx ? wg3 : none, dW_down ? h3 : none}, st);
+    }
+    if (e != cudaSuccess) return cuda_fail(e);
+    if (dW_gate || dx) dh.G3 = dg3.p;
+    ProfScope prof("dh_gemm", st);
+    e = split_gemm(T, F, d, dy3, false, wd3, true, kEpiDH, dh, st);
+  } else {
     ProfScope prof("dh_gemm", st);
     e = gemm(shape, T, F, d, dy, false, W_down, true, kEpiDH, dh, st);
   }
@@ -306,7 +387,12 @@ int stem_ffn_backward(const stem_shape_t* shape, const void* dy, const void* x, 
   EpiParams gp; gp.out_fp32 = grad_fp32; gp.status = status_of(ws);
   gp.accumulate = (shape->flags & STEM_FLAG_ACCUM_GRADS) != 0;
   gp.sk_scratch = base + w.sk_off; gp.sk_bytes = w.sk_bytes;
-  if (dW_down && dW_gate && use_tc(shape)) {
+  if (split && (dW_down || dW_gate)) {
+    const SplitProduct down = split_product(dy3, h3, dW_down, d, F), gate = split_product(dg3, x3, dW_gate, F, d);
+    ProfScope prof("dw_pair_gemm", st);
+    e = launch_split_gemm(dW_down ? down : gate, dW_down && dW_gate ? gate : SplitProduct{}, T, true, true, kEpiStore, gp, st);
+    if (e != cudaSuccess) return cuda_fail(e);
+  } else if (dW_down && dW_gate && use_tc(shape)) {
     // dW_down[i,j] = sum_t dy[t,i] H[t,j] and dW_gate[j,k] = sum_t dG[t,j] x[t,k] in ONE launch: both
     // contract over the tokens, and their output tiles together fill the SMs (at the 350M shape
     // each has 44 tiles for 74 CTA pairs) with one split tail and one fix-up instead of two
@@ -332,7 +418,8 @@ int stem_ffn_backward(const stem_shape_t* shape, const void* dy, const void* x, 
     EpiParams p; p.out = dx; p.out_fp32 = shape->dtype == STEM_DTYPE_FP32; p.status = status_of(ws);
     p.sk_scratch = base + w.sk_off; p.sk_bytes = w.sk_bytes;
     ProfScope prof("dx_gemm", st);
-    e = gemm(shape, T, d, F, dG, false, W_gate, true, kEpiStore, p, st);
+    e = split ? split_gemm(T, d, F, dg3, false, wg3, true, kEpiStore, p, st)
+              : gemm(shape, T, d, F, dG, false, W_gate, true, kEpiStore, p, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
   return STEM_OK;
@@ -425,20 +512,40 @@ int stem_dagger_forward(const stem_shape_t* shape, const void* x, const int32_t*
     e = launch_tc_gemm_dagger(T, F, d, x, W_gate, W_up, du, st);
     if (e != cudaSuccess) return cuda_fail(e);
   } else {
+    const bool split = use_split(shape);
+    const Operand x3 = operand(ws, w.x3_off, x, T, d), wg3 = operand(ws, w.wg3_off, W_gate, F, d),
+                  wu3 = operand(ws, w.wd3_off, W_up, F, d);
+    if (split) {
+      ProfScope prof("split_operands", st);
+      e = split3({x3, wg3, wu3}, st);
+      if (e != cudaSuccess) return cuda_fail(e);
+    }
     {  // U = x W_up^T + E[ids]: the lookup is added in the up GEMM's epilogue
       EpiParams up;
       up.ids = ids; up.E = E; up.V = shape->V; up.H = U_save; up.status = status_of(ws);
       ProfScope prof("up_gemm", st);
-      e = gemm(shape, T, F, d, x, false, W_up, false, kEpiAdd, up, st);
+      e = split ? split_gemm(T, F, d, x3, false, wu3, false, kEpiAdd, up, st)
+                : gemm(shape, T, F, d, x, false, W_up, false, kEpiAdd, up, st);
     }
     if (e != cudaSuccess) return cuda_fail(e);
     {  // G = x W_gate^T, H = SiLU(G) (.) U: the gate epilogue with U as a [T, d_ff] "table" indexed by position
       EpiParams gate;
       gate.ids = nullptr; gate.E = U_save; gate.V = T; gate.H = H; gate.G = G_save; gate.status = status_of(ws);
+      if (split) gate.H3 = operand(ws, w.h3_off, H, T, F).p;
       ProfScope prof("gate_gemm", st);
-      e = gemm(shape, T, F, d, x, false, W_gate, false, kEpiGate, gate, st);
+      e = split ? split_gemm(T, F, d, x3, false, wg3, false, kEpiGate, gate, st)
+                : gemm(shape, T, F, d, x, false, W_gate, false, kEpiGate, gate, st);
     }
     if (e != cudaSuccess) return cuda_fail(e);
+  }
+  if (use_split(shape)) {   // W_down's parts take the place of W_up's
+    const Operand h3 = operand(ws, w.h3_off, H, T, F), wd3 = operand(ws, w.wd3_off, W_down, d, F);
+    EpiParams down;
+    down.out = y; down.status = status_of(ws);
+    ProfScope prof("down_gemm", st);
+    e = split3({wd3}, st);
+    if (e == cudaSuccess) e = split_gemm(T, d, F, h3, false, wd3, false, kEpiStore, down, st);
+    return e == cudaSuccess ? STEM_OK : cuda_fail(e);
   }
   EpiParams down;
   down.out = y; down.out_fp32 = shape->dtype == STEM_DTYPE_FP32; down.status = status_of(ws);
@@ -475,13 +582,32 @@ int stem_dagger_backward(const stem_shape_t* shape, const void* dy, const void* 
   void* dU = base + w.du_off;
   void* dG = base + w.dg_off;
   cudaError_t e;
+  const bool split = use_split(shape);
+  const Operand dy3 = operand(ws, w.dy3_off, dy, T, d), x3 = operand(ws, w.x3_off, x, T, d),
+                wg3 = operand(ws, w.wg3_off, W_gate, F, d), wd3 = operand(ws, w.wd3_off, W_down, d, F),
+                h3 = operand(ws, w.h3_off, H_save, T, F), dg3 = operand(ws, w.dg3_off, dG, T, F);
+  // once dH has read W_down and dW_down has read H, W_up's and dU's parts take their places
+  const Operand wu3 = operand(ws, w.wd3_off, W_up, F, d), du3 = operand(ws, w.h3_off, dU, T, F);
   {  // dH = dy W_down; dU = dH SiLU(G) (gradient of U = W_up x + E[ids]); dG = dH U SiLU'(G)
     EpiParams dh;
     dh.ids = nullptr; dh.E = U_save; dh.V = T; dh.H = dU; dh.G = dG; dh.Gin = G_save; dh.status = status_of(ws);
     ProfScope prof("dh_gemm", st);
-    e = gemm(shape, T, F, d, dy, false, W_down, true, kEpiDH, dh, st);
+    if (split) {
+      Operand none{};
+      dh.G3 = dg3.p;
+      e = split3({dy3, wd3, x3, wg3, dW_down ? h3 : none}, st);
+      if (e == cudaSuccess) e = split_gemm(T, F, d, dy3, false, wd3, true, kEpiDH, dh, st);
+    } else {
+      e = gemm(shape, T, F, d, dy, false, W_down, true, kEpiDH, dh, st);
+    }
   }
   if (e != cudaSuccess) return cuda_fail(e);
+  auto split_grad = [&](const char* name, void* out, int M, int N, const Operand& A, const Operand& Bm) {
+    EpiParams p; p.out = out; p.status = status_of(ws);
+    p.accumulate = (shape->flags & STEM_FLAG_ACCUM_GRADS) != 0;
+    ProfScope prof(name, st);
+    return split_gemm(M, N, T, A, true, Bm, true, kEpiStore, p, st);
+  };
   auto grad = [&](const char* name, void* out, int M, int N, const void* A, const void* Bm) {
     EpiParams p; p.out = out; p.out_fp32 = grad_fp32; p.status = status_of(ws);
     p.accumulate = (shape->flags & STEM_FLAG_ACCUM_GRADS) != 0;
@@ -489,25 +615,31 @@ int stem_dagger_backward(const stem_shape_t* shape, const void* dy, const void* 
     ProfScope prof(name, st);
     return gemm(shape, M, N, T, A, true, Bm, true, kEpiStore, p, st);   // contraction over the tokens
   };
-  if (dW_down && (e = grad("dw_down_gemm", dW_down, d, F, dy, H_save)) != cudaSuccess) return cuda_fail(e);
+  if (dW_down && (e = split ? split_grad("dw_down_gemm", dW_down, d, F, dy3, h3)
+                            : grad("dw_down_gemm", dW_down, d, F, dy, H_save)) != cudaSuccess) return cuda_fail(e);
   if (dE_rows) {
     ProfScope prof("seg_reduce", st);
     e = launch_segreduce(T, F, shape->dtype, shape->grad_dtype, dU, perm, seg_offsets, n_unique, dE_rows,
                          base + w.part_off, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
-  if (dW_gate && (e = grad("dw_gate_gemm", dW_gate, F, d, dG, x)) != cudaSuccess) return cuda_fail(e);
-  if (dW_up && (e = grad("dw_up_gemm", dW_up, F, d, dU, x)) != cudaSuccess) return cuda_fail(e);
+  if (split && (dW_up || dx) && (e = split3({du3, wu3}, st)) != cudaSuccess) return cuda_fail(e);
+  if (dW_gate && (e = split ? split_grad("dw_gate_gemm", dW_gate, F, d, dg3, x3)
+                            : grad("dw_gate_gemm", dW_gate, F, d, dG, x)) != cudaSuccess) return cuda_fail(e);
+  if (dW_up && (e = split ? split_grad("dw_up_gemm", dW_up, F, d, du3, x3)
+                          : grad("dw_up_gemm", dW_up, F, d, dU, x)) != cudaSuccess) return cuda_fail(e);
   if (dx) {  // dx = dG W_gate + dU W_up: the second product is added onto the first in its epilogue
     EpiParams p; p.out = dx; p.out_fp32 = shape->dtype == STEM_DTYPE_FP32; p.status = status_of(ws);
     {
       ProfScope prof("dx_gemm", st);
-      e = gemm(shape, T, d, F, dG, false, W_gate, true, kEpiStore, p, st);
+      e = split ? split_gemm(T, d, F, dg3, false, wg3, true, kEpiStore, p, st)
+                : gemm(shape, T, d, F, dG, false, W_gate, true, kEpiStore, p, st);
     }
     if (e != cudaSuccess) return cuda_fail(e);
     EpiParams a; a.ids = nullptr; a.E = dx; a.V = T; a.H = dx; a.status = status_of(ws);
     ProfScope prof("dx_up_gemm", st);
-    e = gemm(shape, T, d, F, dU, false, W_up, true, kEpiAdd, a, st);
+    e = split ? split_gemm(T, d, F, du3, false, wu3, true, kEpiAdd, a, st)
+              : gemm(shape, T, d, F, dU, false, W_up, true, kEpiAdd, a, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
   return STEM_OK;

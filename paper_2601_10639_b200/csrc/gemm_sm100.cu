@@ -612,17 +612,7 @@ using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, voi
                               CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
                               CUtensorMapFloatOOBfill);
 
-EncodeFn get_encode_fn() {
-  static EncodeFn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      p = nullptr;
-    return reinterpret_cast<EncodeFn>(p);
-  }();
-  return fn;
-}
+EncodeFn get_encode_fn() { return reinterpret_cast<EncodeFn>(tensor_map_encode_fn()); }
 
 // Row-major bf16 matrix [rows, cols] (cols contiguous); box = 64 columns x box_rows rows.
 bool encode_map(CUtensorMap* map, const void* ptr, int rows, int cols, int box_rows) {
@@ -821,6 +811,18 @@ cudaError_t launch_tc_gemm_token_pair(int K, int M1, int N1, const void* A1, con
   second.M = M2; second.N = N2; second.A = A2; second.B = B2; second.out = out2;
   if (pair) return launch_bn<true, true, kEpiStore, 2>(A1, B1, M1, N1, K, p, second, stream);
   return launch_bn<true, true, kEpiStore, 1>(A1, B1, M1, N1, K, p, second, stream);
+}
+
+void* tensor_map_encode_fn() {
+  static void* fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      p = nullptr;
+    return p;
+  }();
+  return fn;
 }
 
 size_t tc_gemm_scratch_bytes() {

@@ -1,8 +1,6 @@
 // FMA-pipe contraction kernels with the layer's fused epilogues.
 //
-// These carry the fp32 configuration (tensor cores have no true fp32 MMA: kind::tf32
-// rounds inputs to a 10-bit mantissa, which cannot meet a 1e-5 error bound) and serve as
-// a slow cross-check for the bf16 tensor-core kernels (STEM_FLAG_SIMT).
+// A slow cross-check for the tensor-core kernels of both types (STEM_FLAG_SIMT).
 #include "stem_internal.h"
 
 namespace stem {

@@ -1,0 +1,695 @@
+// fp32 contraction on the 5th-generation tensor cores, with the layer's elementwise work fused into
+// the epilogue.
+//
+//   C[m,n] = sum_k A(m,k) B(n,k)          A, B, C fp32
+//
+// The tensor cores have no fp32 product, but every fp32 number is the sum of three bf16 numbers
+// (24 = 3 x 8 significand bits): x = x0 + x1 + x2 with x0 = bf16(x), x1 = bf16(x - x0),
+// x2 = x - x0 - x1, every subtraction exact.  A product needs the six terms down to 2^-24 of it:
+// x0 y0, x0 y1, x1 y0, x1 y1, x0 y2, x2 y0 (each a bf16 x bf16 product, exact in fp32).  What the
+// FMA pipes do with 2 flops this does with 12 on a pipe thirty times as fast.
+//
+// Precision.  The tensor core does not round its fp32 accumulation to nearest, so long chains on it
+// drift.  Each 64-wide k block is therefore a sum of its own in tensor memory: the five small terms
+// first, the four x0 y0 instructions last, so that no more than four truncations act on a number of
+// the block sum's size; the block sums are added in fp32 registers, rounded to nearest.  A result
+// that is not finite (an input near the top of the range or not finite: its parts then hold infinities
+// of both signs) or below 2^-98 (third parts below 2^-133 are lost, an error of up to K 2^-134 times
+// the other operand) is computed again from the fp32 operands as one chain of FMAs in ascending k.
+//
+// The parts come from split3_kernel, one launch for all operands of a call, or from the epilogue that
+// produced the operand (EpiParams::H3, G3).  Splitting inside the contraction instead, on the way from
+// global to shared memory, converts every operand once per tile row or column that uses it and is bound
+// by that.  Measured, a layer's training step at 2048 positions, d_model 1024, d_ff 2816: 3600 us on the
+// FMA kernel, 787 us splitting inside, 531 us so (down, dx 63 us = 187 TFLOP/s each; gate 111, dH 128,
+// the weight gradients 126); at 256 positions, 256, 688: 237, 72 and 80 us.  Error against 64 bits:
+// 0.2 - 0.5 of the FMA kernel's for K >= 128, alike at K = 8.
+//
+// A tile is 128 * CTAS rows x BN columns.  CTAS = 2: a pair of CTAs shares each MMA (cta_group::2), each
+// staging its 128 rows of A and half of the columns of B.  Roles per CTA: warp 0 one thread loads with
+// TMA (one copy brings the three parts of a block), warp 1 allocates tensor memory and (first CTA of a
+// pair) issues the 24 MMAs of a block, warps 2..9 add each finished block sum to their registers (one
+// row per thread, two warps per TMEM lane quarter, each half of the columns) and run the epilogue.
+//
+// Bound: shared-memory bandwidth and MMA rate nearly alike.  Per 64-wide block of a pair's tile each CTA
+// is written 72 KB and the MMAs read 144 KB of it, 1730 cycles at 128 bytes a clock, for 1536 cycles of
+// MMA.
+//
+// A launch that would leave SMs idle is cut along k over the CTAs (pairs) of a cluster: each leaves its
+// sums in its own shared memory, and each then adds one share of the columns over the cluster in
+// ascending k.
+#include <cuda.h>
+
+#include "ptx_sm100.cuh"
+#include "stem_internal.h"
+
+namespace stem {
+namespace {
+
+constexpr int BM = 128;
+constexpr int BK = 64;
+constexpr int kAccWarps = 8;
+constexpr int kThreads = 32 * (2 + kAccWarps);
+constexpr long long kWaitLimitCycles = 2000000000ll;  // ~1 s at boost clock
+
+template <int BN, int CTAS>
+struct Smem {
+  static constexpr int kStages = 3;
+  static constexpr int kBCols = BN / CTAS;           // columns of B staged by one CTA
+  static_assert(kBCols == 64, "B is one 64-wide swizzled block per part");
+  static constexpr int kAPart = BM * BK * 2;
+  static constexpr int kBPart = kBCols * BK * 2;
+  static constexpr int kStageBytes = 3 * (kAPart + kBPart);
+  static constexpr int kBarOffset = kStages * kStageBytes;
+  // Block sums in flight in tensor memory: the epilogue of a tile holds the accumulating warps up for
+  // several blocks' time, during which the MMAs go on with the next tile.
+  static constexpr int kBufs = 4;
+  static constexpr int kNumBars = 2 * kStages + 2 * kBufs + 1;   // full, empty, tmem_full, tmem_empty, drain
+  static constexpr int kTotal = kBarOffset + kNumBars * 8 + 16 + 1024;  // + alignment slack
+  static_assert(kTotal <= 232448, "exceeds the shared memory a CTA can have");
+  static_assert(BM * BN * 4 <= kBarOffset, "a tile of fp32 sums must fit the operand ring");
+};
+
+// ---- the three parts ------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+// Two fp32 values -> the packed pairs of their first, second and third parts.
+__device__ __forceinline__ void split_pair(float a, float b, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
+  p0 = pack2(a, b);
+  const float ra = a - __uint_as_float(p0 << 16), rb = b - __uint_as_float(p0 & 0xFFFF0000u);
+  p1 = pack2(ra, rb);
+  p2 = pack2(ra - __uint_as_float(p1 << 16), rb - __uint_as_float(p1 & 0xFFFF0000u));
+}
+
+struct SplitList {
+  SplitJob job[kMaxSplitJobs];
+  int first_block[kMaxSplitJobs + 1];   // blocks [first_block[i], first_block[i + 1]) work on job i
+  int n;
+};
+constexpr int kSplitThreads = 256, kSplitPieces = 2;   // 8-column pieces per thread
+
+// fp32 [rows, cols] -> bf16 [3][rows, pitch], pitch = cols rounded up to 8.  Bound by memory: 4 bytes
+// read and 6 written per element, every access a whole vector of its row.
+__global__ void __launch_bounds__(kSplitThreads) split3_kernel(const __grid_constant__ SplitList list) {
+  ptx::grid_dependency_wait();
+  ptx::grid_launch_dependents();
+  int j = 0;
+  while (j + 1 < list.n && static_cast<int>(blockIdx.x) >= list.first_block[j + 1]) ++j;
+  const SplitJob& job = list.job[j];
+  const int per_row = job.parts.pitch / 8;
+  const long long pieces = static_cast<long long>(job.parts.rows) * per_row;
+  const long long p0 = static_cast<long long>(blockIdx.x - list.first_block[j]) * (kSplitThreads * kSplitPieces) + threadIdx.x;
+  const size_t plane = static_cast<size_t>(job.parts.rows) * job.parts.pitch;
+  float4 v[kSplitPieces][2];
+#pragma unroll
+  for (int i = 0; i < kSplitPieces; ++i) {
+    const long long p = p0 + i * kSplitThreads;
+    v[i][0] = v[i][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (p >= pieces) continue;
+    const float* src = job.src + p * 8;
+    bool whole = true;                     // all eight columns exist
+    if (job.parts.cols != job.parts.pitch) {
+      const long long row = p / per_row;
+      const int c = static_cast<int>(p - row * per_row) * 8;
+      src = job.src + static_cast<size_t>(row) * job.parts.cols + c;
+      whole = c + 4 < job.parts.cols;
+    }
+    v[i][0] = __ldg(reinterpret_cast<const float4*>(src));
+    if (whole) v[i][1] = __ldg(reinterpret_cast<const float4*>(src + 4));
+  }
+#pragma unroll
+  for (int i = 0; i < kSplitPieces; ++i) {
+    const long long p = p0 + i * kSplitThreads;
+    if (p >= pieces) continue;
+    uint4 o[3];
+    split_pair(v[i][0].x, v[i][0].y, o[0].x, o[1].x, o[2].x);
+    split_pair(v[i][0].z, v[i][0].w, o[0].y, o[1].y, o[2].y);
+    split_pair(v[i][1].x, v[i][1].y, o[0].z, o[1].z, o[2].z);
+    split_pair(v[i][1].z, v[i][1].w, o[0].w, o[1].w, o[2].w);
+    __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(job.parts.base) + p * 8;
+#pragma unroll
+    for (int s = 0; s < 3; ++s) *reinterpret_cast<uint4*>(dst + s * plane) = o[s];
+  }
+}
+
+// ---- epilogue ---------------------------------------------------------------------------------
+// One product of the launch.  A second one with the same K and layouts may ride along (plain stores
+// only); its tiles are numbered after the first one's.
+struct Product {
+  const float* A = nullptr;      // the fp32 operands, for results that the parts cannot carry
+  const float* B = nullptr;
+  float* out = nullptr;
+  int M = 0, N = 0;
+  bool wide = false;             // 32-byte accesses are legal in every [., N] matrix of the epilogue
+};
+
+// Results that the parts cannot carry: not finite, or so small that the third parts of the inputs fell
+// below bf16's smallest number.  Zero is what it is.
+__device__ __forceinline__ bool needs_chain(float v) {
+  const uint32_t u = __float_as_uint(v) & 0x7FFFFFFFu;
+  constexpr uint32_t kTiny = 29u << 23;   // 2^-98
+  return u - kTiny > 0x7F7FFFFFu - kTiny && u != 0;
+}
+// The plain chain of FMAs for them; a[i] is column n + i of row m.  (One loop over the marked columns:
+// a copy of the chain per column would be most of the kernel's code.  A NaN stays one, so the chain
+// ends there.)
+template <bool A_MN, bool B_MN>
+__device__ __forceinline__ void redo_in_fp32(const Product& pr, int K, int m, int n, float (&a)[32]) {
+  uint32_t marked = 0;
+#pragma unroll
+  for (int i = 0; i < 32; ++i)
+    if (needs_chain(a[i]) && n + i < pr.N) marked |= 1u << i;
+  while (marked != 0) {
+    const int i = __ffs(marked) - 1;
+    marked &= marked - 1;
+    float acc = 0.0f;
+#pragma unroll 1
+    for (int k = 0; k < K && acc == acc; ++k)
+      acc = fmaf(A_MN ? pr.A[static_cast<size_t>(k) * pr.M + m] : pr.A[static_cast<size_t>(m) * K + k],
+                 B_MN ? pr.B[static_cast<size_t>(k) * pr.N + n + i] : pr.B[static_cast<size_t>(n + i) * K + k], acc);
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (j == i) a[j] = acc;
+  }
+}
+
+// Eight consecutive values of a row; WIDE: the row pitch and the base are multiples of 32 bytes.
+// have: how many of them exist (a multiple of 4, at most 8).  Plain loads: kEpiAdd may overwrite its addend.
+__device__ __forceinline__ void load8(const float* p, bool wide, int have, float* x) {
+  if (wide && have >= 8) {
+    asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7])
+                 : "l"(p) : "memory");
+    return;
+  }
+#pragma unroll
+  for (int h = 0; h < 8; h += 4) {
+    if (h < have) {
+      const float4 q = *reinterpret_cast<const float4*>(p + h);
+      x[h] = q.x; x[h + 1] = q.y; x[h + 2] = q.z; x[h + 3] = q.w;
+    }
+  }
+}
+__device__ __forceinline__ void store8(float* p, bool wide, int have, const float (&x)[8]) {
+  if (wide && have >= 8) {
+    asm volatile("st.global.v8.f32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};"
+                 ::"f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "f"(x[4]), "f"(x[5]), "f"(x[6]), "f"(x[7]), "l"(p)
+                 : "memory");
+    return;
+  }
+#pragma unroll
+  for (int h = 0; h < 8; h += 4)
+    if (h < have) *reinterpret_cast<float4*>(p + h) = make_float4(x[h], x[h + 1], x[h + 2], x[h + 3]);
+}
+__device__ __forceinline__ void store_parts8(const Parts& parts, int m, int n, int have, const float (&r)[8]) {
+  uint32_t o[3][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) split_pair(r[2 * i], r[2 * i + 1], o[0][i], o[1][i], o[2][i]);
+  __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(parts.base) + static_cast<size_t>(m) * parts.pitch + n;
+  const size_t plane = static_cast<size_t>(parts.rows) * parts.pitch;
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    if (have >= 8) *reinterpret_cast<uint4*>(dst + s * plane) = make_uint4(o[s][0], o[s][1], o[s][2], o[s][3]);
+    else *reinterpret_cast<uint2*>(dst + s * plane) = make_uint2(o[s][0], o[s][1]);
+  }
+}
+
+// The operands that the fused step needs for 32 consecutive columns (n_cols of which are this thread's)
+// of one row: the table row (or addend) and the saved G.
+template <int KIND>
+__device__ __forceinline__ void load_operands(const EpiParams& ep, const Product& pr, int m, int n, int n_cols, int row_id,
+                                              float (&e)[32], float (&g)[32]) {
+  if (KIND == kEpiStore) return;
+  const float* e_row = static_cast<const float*>(ep.E) + static_cast<size_t>(row_id) * pr.N + n;
+  const float* g_row = static_cast<const float*>(ep.Gin) + static_cast<size_t>(m) * pr.N + n;
+#pragma unroll
+  for (int c = 0; c < 32; c += 8) {
+    const int have = min(n_cols, pr.N - n) - c;
+    if (have > 0) {
+      load8(e_row + c, pr.wide, have, e + c);
+      if (KIND == kEpiDH) load8(g_row + c, pr.wide, have, g + c);
+    }
+  }
+}
+
+// Fused elementwise step on them (formulas: EpiParams).
+template <int KIND>
+__device__ __forceinline__ void epilogue32(const EpiParams& ep, const Product& pr, int m, int n, int n_cols,
+                                           const float (&a)[32], const float (&e)[32], const float (&g)[32]) {
+#pragma unroll
+  for (int c = 0; c < 32; c += 8) {
+    const int have = min(n_cols, pr.N - n) - c;
+    if (have <= 0) break;
+    const size_t o = static_cast<size_t>(m) * pr.N + n + c;
+    float r[8], r2[8];
+    if (KIND == kEpiStore && ep.accumulate) {
+      load8(pr.out + o, pr.wide, have, r2);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float x = a[c + i];
+      if (KIND == kEpiStore) {
+        r[i] = ep.accumulate ? x + r2[i] : x;
+      } else if (KIND == kEpiAdd) {
+        r[i] = x + e[c + i];
+      } else if (KIND == kEpiGate) {
+        r[i] = x * sigmoid_f32(x) * e[c + i];
+        r2[i] = x;
+      } else {
+        const float gi = g[c + i], s = sigmoid_f32(gi);
+        r[i] = x * (gi * s);                                       // dU
+        r2[i] = x * e[c + i] * (s * (1.0f + gi * (1.0f - s)));     // dG
+      }
+    }
+    store8((KIND == kEpiStore ? pr.out : static_cast<float*>(ep.H)) + o, pr.wide, have, r);
+    if (KIND == kEpiGate && ep.H3.base != nullptr) store_parts8(ep.H3, m, n + c, have, r);
+    if (KIND == kEpiDH || (KIND == kEpiGate && ep.G != nullptr)) store8(static_cast<float*>(ep.G) + o, pr.wide, have, r2);
+    if (KIND == kEpiDH && ep.G3.base != nullptr) store_parts8(ep.G3, m, n + c, have, r2);
+  }
+}
+
+template <int KIND>
+__device__ __forceinline__ int table_row(const EpiParams& ep, int m) {
+  if (KIND == kEpiStore) return 0;
+  int id = ep.ids != nullptr ? ep.ids[m] : m;
+  if (id < 0 || id >= ep.V) {
+    report_error(ep.status, STEM_ERR_ID_RANGE, m);
+    id = id < 0 ? 0 : ep.V - 1;
+  }
+  return id;
+}
+
+// ---- the contraction ----------------------------------------------------------------------------
+struct Maps { CUtensorMap A, B, A2, B2; };   // [3][rows, cols] parts; the second product's
+
+template <bool A_MN, bool B_MN, int KIND, int BN, int CTAS>
+__global__ void __launch_bounds__(kThreads, 1)
+split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Product p1,
+                  const __grid_constant__ Product p2, int K, int ksplit, const __grid_constant__ EpiParams ep) {
+  using L = Smem<BN, CTAS>;
+  constexpr int STAGES = L::kStages;
+  constexpr int TM = BM * CTAS;
+  constexpr int BUFS = L::kBufs;
+  constexpr uint32_t kTmemCols = BUFS * BN;
+  static_assert(kTmemCols <= 512, "tensor memory has 512 columns");
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = ptx::smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t* base_ptr = smem_raw + (base - raw);
+  const uint32_t bars = base + L::kBarOffset;
+  auto full_bar = [&](int s) { return bars + 8u * s; };
+  auto empty_bar = [&](int s) { return bars + 8u * (STAGES + s); };
+  auto tfull_bar = [&](int a) { return bars + 8u * (2 * STAGES + a); };
+  auto tempty_bar = [&](int a) { return bars + 8u * (2 * STAGES + BUFS + a); };
+  const uint32_t drain_bar = bars + 8u * (2 * STAGES + 2 * BUFS);
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + L::kBarOffset + L::kNumBars * 8);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + L::kBarOffset + L::kNumBars * 8 + 4);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool clustered = CTAS * ksplit > 1;
+  const uint32_t crank = clustered ? ptx::cluster_ctarank() : 0u;
+  const uint32_t rank = CTAS == 2 ? crank & 1u : 0u;              // inside the pair
+  const uint32_t leader = crank - rank;
+  const uint16_t pair_mask = static_cast<uint16_t>(3u << leader);
+  const int tiles_m1 = (p1.M + TM - 1) / TM, tiles1 = tiles_m1 * ((p1.N + BN - 1) / BN);
+  const int tiles_m2 = (p2.M + TM - 1) / TM, tiles2 = tiles_m2 * ((p2.N + BN - 1) / BN);
+  const int num_tiles = tiles1 + tiles2;
+  const int k_blocks = (K + BK - 1) / BK;
+  // ksplit > 1: the launch has one cluster per tile, and each CTA (pair) of it a k range
+  const int slice = static_cast<int>(crank) / CTAS;
+  const int tile0 = blockIdx.x / (CTAS * ksplit), tile_step = gridDim.x / (CTAS * ksplit);
+  const int kb0 = static_cast<int>(static_cast<long long>(k_blocks) * slice / ksplit);
+  const int kb1 = static_cast<int>(static_cast<long long>(k_blocks) * (slice + 1) / ksplit);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) { ptx::mbar_init(full_bar(s), 1); ptx::mbar_init(empty_bar(s), 1); }
+    for (int a = 0; a < BUFS; ++a) { ptx::mbar_init(tfull_bar(a), 1); ptx::mbar_init(tempty_bar(a), kAccWarps * CTAS); }
+    ptx::mbar_init(drain_bar, 1);
+    *abort_flag = 0;
+    ptx::fence_mbar_init();
+    ptx::prefetch_tensormap(&maps.A);
+    ptx::prefetch_tensormap(&maps.B);
+    if (KIND == kEpiStore && tiles2 > 0) { ptx::prefetch_tensormap(&maps.A2); ptx::prefetch_tensormap(&maps.B2); }
+  }
+  if (warp == 1) {
+    if (CTAS == 2) {
+      ptx::tmem_alloc_pair(ptx::smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
+      ptx::tmem_relinquish_pair();
+    } else {
+      ptx::tmem_alloc(ptx::smem_u32(const_cast<uint32_t*>(tmem_slot)), kTmemCols);
+      ptx::tmem_relinquish();
+    }
+  }
+  ptx::tc_fence_before();
+  if (clustered) ptx::cluster_sync(); else __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  ptx::grid_dependency_wait();
+  ptx::grid_launch_dependents();
+
+  int issued = 0;   // producer: blocks handed to TMA so far
+  bool ok = true;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int s = 0; uint32_t ph = 0;
+      for (int tile = tile0; ok && tile < num_tiles; tile += tile_step) {
+        const bool second = KIND == kEpiStore && tile >= tiles1;
+        const CUtensorMap* mapA = second ? &maps.A2 : &maps.A;
+        const CUtensorMap* mapB = second ? &maps.B2 : &maps.B;
+        const int tt = second ? tile - tiles1 : tile, tm = second ? tiles_m2 : tiles_m1;
+        const int m0 = tt % tm * TM + rank * BM, n0 = tt / tm * BN + rank * L::kBCols;
+        for (int kb = kb0; kb < kb1; ++kb) {
+          if (!ptx::mbar_wait_bounded(empty_bar(s), ph ^ 1u, abort_flag, kWaitLimitCycles)) {
+            report_error(ep.status, STEM_ERR_TIMEOUT, 1);
+            *abort_flag = 1; ok = false; break;
+          }
+          const uint32_t a_dst = base + s * L::kStageBytes, b_dst = a_dst + 3 * L::kAPart;
+          // the first CTA of a pair waits on its own barrier for the bytes of both
+          if (rank == 0) ptx::mbar_arrive_expect_tx(full_bar(s), CTAS * L::kStageBytes);
+          const uint32_t fb = CTAS == 2 ? ptx::mapa(full_bar(s), leader) : full_bar(s);
+          auto load = [&](uint32_t dst, const CUtensorMap* map, int c0, int c1) {
+            if (CTAS == 2) ptx::tma_load_3d_pair(dst, map, fb, c0, c1, 0); else ptx::tma_load_3d(dst, map, fb, c0, c1, 0);
+          };
+          const int k0 = kb * BK;
+          // K-major: [part][128 rows][64 k].  MN-major: two 64-wide blocks, each [part][64 k][64 m].
+          if (A_MN) {
+            load(a_dst, mapA, m0, k0);
+            load(a_dst + 3 * L::kAPart / 2, mapA, m0 + 64, k0);
+          } else {
+            load(a_dst, mapA, k0, m0);
+          }
+          if (B_MN) load(b_dst, mapB, n0, k0); else load(b_dst, mapB, k0, n0);
+          ++issued;
+          if (++s == STAGES) { s = 0; ph ^= 1u; }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0 && rank == 0) {
+      constexpr uint32_t idesc = ptx::make_idesc_bf16(TM, BN, A_MN, B_MN);
+      auto commit = [&](uint32_t bar) { if (CTAS == 2) ptx::mma_commit_pair(bar, pair_mask); else ptx::mma_commit(bar); };
+      int s = 0; uint32_t ph = 0;
+      int acc = 0; uint32_t aph = 0;
+      for (int tile = tile0; ok && tile < num_tiles; tile += tile_step) {
+        for (int kb = kb0; kb < kb1; ++kb) {
+          if (!ptx::mbar_wait_bounded(tempty_bar(acc), aph ^ 1u, abort_flag, kWaitLimitCycles) ||
+              !ptx::mbar_wait_bounded(full_bar(s), ph, abort_flag, kWaitLimitCycles)) {
+            report_error(ep.status, STEM_ERR_TIMEOUT, 2);
+            *abort_flag = 1; ok = false; break;
+          }
+          ptx::tc_fence_after();
+          const uint32_t d_tmem = tmem_base + acc * BN;
+          const uint32_t a_src = base + s * L::kStageBytes, b_src = a_src + 3 * L::kAPart;
+          constexpr int kTerms = 6;
+          constexpr int ia[kTerms] = {2, 0, 1, 1, 0, 0}, ib[kTerms] = {0, 2, 1, 0, 1, 0};   // smallest terms first
+          // bytes from one part of A to the next, and (MN-major) from one 64-wide block to the next
+          constexpr int a_part = A_MN ? L::kAPart / 2 : L::kAPart, a_block = 3 * L::kAPart / 2;
+#pragma unroll
+          for (int term = 0; term < kTerms; ++term) {
+#pragma unroll
+            for (int kk = 0; kk < BK / 16; ++kk) {
+              const uint32_t a = a_src + ia[term] * a_part, b = b_src + ib[term] * L::kBPart;
+              const uint64_t ad = A_MN ? ptx::make_smem_desc(a + kk * (16 * 128), a_block, 1024)
+                                       : ptx::make_smem_desc(a + kk * 32, 16, 1024);
+              const uint64_t bd = B_MN ? ptx::make_smem_desc(b + kk * (16 * 128), L::kBPart, 1024)
+                                       : ptx::make_smem_desc(b + kk * 32, 16, 1024);
+              if (CTAS == 2) ptx::mma_bf16_ss_pair(d_tmem, ad, bd, idesc, (term > 0 || kk > 0) ? 1u : 0u);
+              else ptx::mma_bf16_ss(d_tmem, ad, bd, idesc, (term > 0 || kk > 0) ? 1u : 0u);
+            }
+          }
+          commit(empty_bar(s));
+          commit(tfull_bar(acc));
+          if (++s == STAGES) { s = 0; ph ^= 1u; }
+          if (++acc == BUFS) { acc = 0; aph ^= 1u; }
+        }
+      }
+      if (!ok) {
+        // let MMAs already issued finish before TMEM is freed
+        if (CTAS == 2) ptx::mma_commit_pair(drain_bar, static_cast<uint16_t>(1u << leader)); else ptx::mma_commit(drain_bar);
+        int zero = 0;
+        ptx::mbar_wait_bounded(drain_bar, 0, &zero, kWaitLimitCycles);
+      }
+    }
+  } else {
+    constexpr int kCols = BN / 2;           // columns per thread
+    const int q = warp & 3;                 // TMEM lane quarter this warp may read
+    const int half = (warp - 2) >> 2;       // which half of the tile's columns it handles
+    const int r = q * 32 + lane;            // row among this CTA's 128
+    int buf = 0; uint32_t bph = 0;
+    float acc[kCols / 32][32], e[32], g[32];
+    const int share = kCols / ksplit;       // columns of a tile that this thread finishes
+    int id = 0;
+    for (int tile = tile0; ok && tile < num_tiles; tile += tile_step) {
+      const bool second = KIND == kEpiStore && tile >= tiles1;
+      const Product& pr = second ? p2 : p1;
+      const int tt = second ? tile - tiles1 : tile, tm = second ? tiles_m2 : tiles_m1;
+      const int m = tt % tm * TM + rank * BM + r, n0 = tt / tm * BN + half * kCols;
+#pragma unroll
+      for (int c = 0; c < kCols; ++c) acc[c / 32][c % 32] = 0.0f;
+      // the epilogue's first operands are on their way while the blocks are summed
+      if (KIND != kEpiStore && m < pr.M) {
+        id = table_row<KIND>(ep, m);
+        load_operands<KIND>(ep, pr, m, n0 + slice * share, share, id, e, g);
+      }
+      for (int kb = kb0; kb < kb1; ++kb) {
+        bool mine = ptx::mbar_wait_bounded(tfull_bar(buf), bph, abort_flag, kWaitLimitCycles);
+        if (!__all_sync(0xffffffffu, mine)) {
+          if (lane == 0) { report_error(ep.status, STEM_ERR_TIMEOUT, 4); *abort_flag = 1; }
+          ok = false; break;
+        }
+        ptx::tc_fence_after();
+        const uint32_t t_row = tmem_base + buf * BN + half * kCols + (static_cast<uint32_t>(q * 32) << 16);
+#pragma unroll
+        for (int c = 0; c < kCols; c += 32) {
+          uint32_t v[32];
+          ptx::tmem_ld_32x32(t_row + c, v);
+          ptx::tmem_ld_wait();
+          if (c + 32 == kCols) {   // read out: the buffer goes back to the MMA issuer
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) {
+              if (rank == 0) ptx::mbar_arrive(tempty_bar(buf));
+              else ptx::mbar_arrive_cluster(ptx::mapa(tempty_bar(buf), leader));
+            }
+          }
+#pragma unroll
+          for (int i = 0; i < 32; ++i) acc[c / 32][i] += __uint_as_float(v[i]);
+        }
+        if (++buf == BUFS) { buf = 0; bph ^= 1u; }
+      }
+      if (!ok) break;
+      if (ksplit == 1) {
+        if (m < pr.M) {
+#pragma unroll
+          for (int c = 0; c < kCols; c += 32) {
+            if (c > 0) load_operands<KIND>(ep, pr, m, n0 + c, 32, id, e, g);
+            redo_in_fp32<A_MN, B_MN>(pr, K, m, n0 + c, acc[c / 32]);
+            epilogue32<KIND>(ep, pr, m, n0 + c, 32, acc[c / 32], e, g);
+          }
+        }
+      } else {
+        // This CTA's copies have landed and its MMAs (a pair's: of both) are complete, so the operand
+        // ring is free: leave the sums there, column by column (128 rows of a column side by side).
+        float* part = reinterpret_cast<float*>(base_ptr) + static_cast<size_t>(half) * kCols * BM + r;
+#pragma unroll
+        for (int c = 0; c < kCols; ++c) part[c * BM] = acc[c / 32][c % 32];
+      }
+    }
+    if (ksplit > 1) {
+      // Every thread of every CTA of the cluster meets this barrier, also after a timeout.
+      __syncwarp();
+      ptx::cluster_sync();
+      const bool second = KIND == kEpiStore && tile0 >= tiles1;
+      const Product& pr = second ? p2 : p1;
+      const int tt = second ? tile0 - tiles1 : tile0, tm = second ? tiles_m2 : tiles_m1;
+      const int m = tt % tm * TM + rank * BM + r, n0 = tt / tm * BN + half * kCols + slice * share;
+      if (ok && m < pr.M) {
+        const uint32_t mine = base + 4u * (static_cast<uint32_t>(half * kCols + slice * share) * BM + r);
+        float v[32];
+#pragma unroll
+        for (int c = 0; c < 32; ++c) v[c] = 0.0f;
+        for (int k = 0; k < ksplit; ++k) {
+          const uint32_t src = ptx::mapa(mine, k * CTAS + rank);
+#pragma unroll
+          for (int c = 0; c < 32; ++c)
+            if (c < share) v[c] += ptx::ld_shared_cluster_f32(src + 4u * BM * c);
+        }
+        redo_in_fp32<A_MN, B_MN>(pr, K, m, n0, v);
+        epilogue32<KIND>(ep, pr, m, n0, share, v, e, g);
+      }
+      __syncwarp();
+    }
+  }
+
+  if (ksplit > 1 && warp < 2) { __syncwarp(); ptx::cluster_sync(); }   // (the other warps': above)
+  __syncwarp();
+  __syncthreads();
+  if (*abort_flag != 0 && threadIdx.x == 0) {
+    // wait (bounded) for copies still in flight; the second CTA of a pair cannot poll the barriers
+    // its bytes are counted on and waits out a fixed interval (far longer than a copy takes)
+    int zero = 0;
+    if (rank == 0) {
+      for (int j = issued > STAGES ? issued - STAGES : 0; j < issued; ++j)
+        ptx::mbar_wait_bounded(full_bar(j % STAGES), (j / STAGES) & 1, &zero, kWaitLimitCycles / 16);
+    } else {
+      const long long t0 = clock64();
+      while (clock64() - t0 < 2000000ll) { }
+    }
+  }
+  // No CTA of a cluster leaves (or frees TMEM) while another can still signal its barriers, read its
+  // shared memory or write its accumulators.
+  if (clustered) ptx::cluster_sync(); else __syncthreads();
+  if (warp == 1) {
+    ptx::tc_fence_after();
+    if (CTAS == 2) ptx::tmem_dealloc_pair(tmem_base, kTmemCols); else ptx::tmem_dealloc(tmem_base, kTmemCols);
+  }
+}
+
+// ---- host side -------------------------------------------------------------------------------
+// Parts [3][rows, cols] with a row pitch; box = 64 columns x box_rows rows x all three parts.
+bool encode_parts(CUtensorMap* map, const Parts& p, int box_rows) {
+  const auto fn = reinterpret_cast<CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                                const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
+                                                CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
+                                                CUtensorMapFloatOOBfill)>(tensor_map_encode_fn());
+  if (!fn) return false;
+  const cuuint64_t dims[3] = {static_cast<cuuint64_t>(p.cols), static_cast<cuuint64_t>(p.rows), 3u};
+  const cuuint64_t strides[2] = {static_cast<cuuint64_t>(p.pitch) * 2, static_cast<cuuint64_t>(p.pitch) * 2 * p.rows};
+  const cuuint32_t box[3] = {64u, static_cast<cuuint32_t>(box_rows), 3u};
+  const cuuint32_t estr[3] = {1u, 1u, 1u};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, p.base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Tile shape and k split.  The time of a launch is its rounds of tiles over the SMs times the k blocks of
+// a tile times a block's cost (1750 cycles for either shape, by shared-memory bytes; a pair's tile is
+// four times as large on twice the SMs), plus a tile's own latencies, plus what adding the slices
+// costs.  A cluster has at most 8 CTAs, and a slice at least 2 blocks.
+struct Plan { bool pair; int ksplit; };
+long long tile_count(int M, int N, int tm, int bn) { return static_cast<long long>((M + tm - 1) / tm) * ((N + bn - 1) / bn); }
+Plan make_plan(int M1, int N1, int M2, int N2, int K) {
+  const int k_blocks = (K + BK - 1) / BK;
+  Plan best{true, 1};
+  double best_cost = 0.0;
+  for (bool pair : {true, false}) {
+    const int ctas = pair ? 2 : 1, slots = device_sm_count() / ctas;
+    const long long tiles = tile_count(M1, N1, BM * ctas, 64 * ctas) + tile_count(M2, N2, BM * ctas, 64 * ctas);
+    for (int sp = 1; sp * ctas <= 8; sp *= 2) {
+      if (sp > 1 && (tiles * sp > slots || k_blocks < 2 * sp)) break;
+      const double rounds = static_cast<double>((tiles * sp + slots - 1) / slots);
+      const double cost = rounds * ((k_blocks + sp - 1) / sp * 1750.0) + 3000.0 + (sp > 1 ? 2500.0 : 0.0);
+      if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = {pair, sp}; }
+    }
+  }
+  return best;
+}
+
+template <bool A_MN, bool B_MN, int KIND, int CTAS>
+cudaError_t launch_inst(const SplitProduct& a, const SplitProduct& b, int K, int ksplit, const EpiParams& ep,
+                        cudaStream_t stream) {
+  constexpr int BN = 64 * CTAS;
+  using L = Smem<BN, CTAS>;
+  auto kern = split_gemm_kernel<A_MN, B_MN, KIND, BN, CTAS>;
+  static PerDeviceOnce configured;
+  if (cudaError_t ce = configured.run([&] {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kTotal);
+      }))
+    return ce;
+  Maps maps;
+  const int rows_a = A_MN ? BK : BM, rows_b = 64;
+  bool good = encode_parts(&maps.A, a.A3, rows_a) && encode_parts(&maps.B, a.B3, rows_b);
+  if (b.M > 0) good = good && encode_parts(&maps.A2, b.A3, rows_a) && encode_parts(&maps.B2, b.B3, rows_b);
+  else { maps.A2 = maps.A; maps.B2 = maps.B; }
+  if (!good) return cudaErrorNotSupported;
+  Product p[2];
+  const SplitProduct* src[2] = {&a, &b};
+  auto a32 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 31u) == 0; };
+  for (int i = 0; i < 2; ++i) {
+    const bool wide = src[i]->N % 8 == 0 && a32(src[i]->out) && a32(ep.E) && a32(ep.Gin) && a32(ep.H) && a32(ep.G);
+    p[i] = {src[i]->A, src[i]->B, src[i]->out, src[i]->M, src[i]->N, wide};
+  }
+  const long long tiles = tile_count(a.M, a.N, BM * CTAS, BN) + tile_count(b.M, b.N, BM * CTAS, BN);
+  const int slots = device_sm_count() / CTAS;
+  const long long units = ksplit > 1 ? tiles * ksplit : (tiles < slots ? tiles : slots);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(units * CTAS));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = L::kTotal;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned>(CTAS * ksplit);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = CTAS * ksplit > 1 ? 2 : 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, maps, p[0], p[1], K, ksplit, ep);
+  count_launches(1);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <bool A_MN, bool B_MN, int KIND>
+cudaError_t launch_planned(const SplitProduct& a, const SplitProduct& b, int K, const EpiParams& ep, cudaStream_t stream) {
+  const Plan pl = make_plan(a.M, a.N, b.M, b.N, K);
+  if (pl.pair) return launch_inst<A_MN, B_MN, KIND, 2>(a, b, K, pl.ksplit, ep, stream);
+  return launch_inst<A_MN, B_MN, KIND, 1>(a, b, K, pl.ksplit, ep, stream);
+}
+
+}  // namespace
+
+cudaError_t launch_split3(const SplitJob* jobs, int n, cudaStream_t stream) {
+  SplitList list;
+  list.n = 0;
+  long long blocks = 0;
+  for (int i = 0; i < n; ++i) {
+    const Parts& p = jobs[i].parts;
+    if (p.rows <= 0 || p.cols <= 0) continue;
+    if (list.n == kMaxSplitJobs || p.cols % 4) return cudaErrorNotSupported;
+    list.job[list.n] = jobs[i];
+    list.first_block[list.n++] = static_cast<int>(blocks);
+    const long long pieces = static_cast<long long>(p.rows) * (p.pitch / 8), per_block = kSplitThreads * kSplitPieces;
+    blocks += (pieces + per_block - 1) / per_block;
+  }
+  if (list.n == 0) return cudaSuccess;
+  if (blocks > 0x7fffffffll) return cudaErrorNotSupported;
+  list.first_block[list.n] = static_cast<int>(blocks);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(blocks));
+  cfg.blockDim = dim3(kSplitThreads);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, split3_kernel, list);
+  count_launches(1);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_split_gemm(const SplitProduct& p, const SplitProduct& second, int K, bool a_mn, bool b_mn, EpiKind kind,
+                              const EpiParams& ep, cudaStream_t stream) {
+  if (p.M <= 0 || p.N <= 0) return cudaSuccess;
+  if (K <= 0 || (p.N % 4) || (second.N % 4)) return cudaErrorNotSupported;
+  // the layer's call sites: gate, up (K,K)  down (K,K,store)  dH, dx (K,MN)  dW_* (MN,MN,store)
+  if (second.M > 0 && !(a_mn && b_mn && kind == kEpiStore)) return cudaErrorNotSupported;
+  if (!a_mn && !b_mn) {
+    if (kind == kEpiGate) return launch_planned<false, false, kEpiGate>(p, second, K, ep, stream);
+    if (kind == kEpiAdd) return launch_planned<false, false, kEpiAdd>(p, second, K, ep, stream);
+    if (kind == kEpiStore) return launch_planned<false, false, kEpiStore>(p, second, K, ep, stream);
+  } else if (!a_mn && b_mn) {
+    if (kind == kEpiDH) return launch_planned<false, true, kEpiDH>(p, second, K, ep, stream);
+    if (kind == kEpiAdd) return launch_planned<false, true, kEpiAdd>(p, second, K, ep, stream);
+    if (kind == kEpiStore) return launch_planned<false, true, kEpiStore>(p, second, K, ep, stream);
+  } else if (a_mn && b_mn) {
+    if (kind == kEpiStore) return launch_planned<true, true, kEpiStore>(p, second, K, ep, stream);
+  }
+  return cudaErrorNotSupported;
+}
+
+}  // namespace stem

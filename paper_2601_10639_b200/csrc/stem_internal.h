@@ -38,6 +38,13 @@ __device__ __forceinline__ float sigmoid_f32(float g) { return 1.0f / (1.0f + ex
 // ---- epilogue descriptions (shared by the FMA and the tensor-core GEMM front ends) ---
 enum EpiKind : int { kEpiStore = 0, kEpiGate = 1, kEpiDH = 2, kEpiAdd = 3, kEpiDagger = 4 };
 
+// An fp32 matrix as the sum of three bf16 ones: [3][rows, cols], row pitch a multiple of 8 elements.
+struct Parts {
+  void* base = nullptr;
+  int rows = 0, cols = 0, pitch = 0;
+};
+inline size_t parts_bytes(size_t rows, size_t cols) { return align_up(3 * rows * ((cols + 7) / 8 * 8) * 2, 256); }
+
 struct EpiParams {
   // kEpiStore: out[m*ld + n] = acc              (out_fp32 selects fp32 or bf16/T storage)
   //            accumulate: out[m*ld + n] += acc   (gradient accumulation over micro-batches)
@@ -58,6 +65,8 @@ struct EpiParams {
   // kEpiDagger (two products of the same A tile, gate = acc and up = acc2):
   //            U = acc2 + E[ids[m], n]; H = SiLU(acc) * U; optional G = acc, optional U out
   void* U = nullptr;
+  // fp32 on the tensor cores, optional: the parts of H (kEpiGate) and of dG (kEpiDH) as well
+  Parts H3, G3;
   int32_t* status = nullptr;
   // kEpiStore, optional: scratch for partial tiles when the last round of tiles is split
   // along k (tc_gemm_scratch_bytes()); without it every tile is computed whole
@@ -70,6 +79,25 @@ struct EpiParams {
 cudaError_t launch_simt_gemm(int dtype, int M, int N, int K, const void* A, bool a_mn,
                              const void* B, bool b_mn, EpiKind kind, const EpiParams& ep,
                              cudaStream_t stream);
+
+// fp32 contraction on the tensor cores, each operand as three bf16 parts (split_gemm.cu).  The caller
+// provides the parts: launch_split3 makes those of up to kMaxSplitJobs matrices in one launch, and the
+// gate / dH epilogues write those of H / dG (EpiParams::H3, G3).
+struct SplitJob { const float* src; Parts parts; };
+constexpr int kMaxSplitJobs = 6;
+cudaError_t launch_split3(const SplitJob* jobs, int n, cudaStream_t stream);
+// Same contraction, layouts and epilogues as below with fp32 storage; extents that are contiguous in
+// memory are multiples of 4, else cudaErrorNotSupported.  `second` (M == 0: none) rides in the same
+// launch: token-contracted plain stores only.
+struct SplitProduct {
+  const float* A = nullptr;
+  const float* B = nullptr;
+  Parts A3, B3;
+  float* out = nullptr;     // kEpiStore
+  int M = 0, N = 0;
+};
+cudaError_t launch_split_gemm(const SplitProduct& p, const SplitProduct& second, int K, bool a_mn, bool b_mn, EpiKind kind,
+                              const EpiParams& ep, cudaStream_t stream);
 
 // tcgen05 / TMEM / TMA kernels, bf16 inputs.  Returns cudaErrorNotSupported when the
 // shape cannot be described to TMA (the caller decides what to do).
@@ -93,6 +121,7 @@ cudaError_t launch_tc_gemm_dagger(int M, int N, int K, const void* A, const void
                                   const EpiParams& ep, cudaStream_t stream);
 
 size_t tc_gemm_scratch_bytes();
+void* tensor_map_encode_fn();   // cuTensorMapEncodeTiled, or NULL
 
 // ---- index path ----------------------------------------------------------------------
 size_t dedup_workspace_bytes(int T, int V);

@@ -1,0 +1,70 @@
+"""fp32 layers on the tensor cores (each operand as three bf16 parts) vs the CPU checker, where the
+kernel can go wrong: extents that end inside a 64-wide block, a row pitch that is a multiple of 4 only,
+one tile and several rounds of tiles, launches cut along k, two products in one launch, inputs that the
+parts cannot carry."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import stem_oracle as O
+from paper_2601_10639_b200 import binding as B
+from paper_2601_10639_b200 import runner, synth
+from parity_measures import TOL_FP32
+from test_gpu_parity import _full_parity, _np
+
+pytestmark = pytest.mark.gpu
+
+
+# TOL_FP32 = 1e-5 is what the fp32 configuration is held to; a chain of K <= 2820 fp32 additions rounds
+# to about sqrt(K) 2^-24 = 3e-6 of its result, K / 64 block sums to less
+@pytest.mark.parametrize("flags", [0, B.FLAG_SIMT], ids=["parts", "fma"])
+@pytest.mark.parametrize("T,d,F", [(1, 8, 12), (65, 68, 132), (131, 260, 644), (300, 64, 136), (777, 700, 1500),
+                                   (1500, 260, 2820)])
+def test_layer_fp32(flags, T, d, F):
+    w = synth.Workload("t", T, d, F, 500, "fp32", "zipf")
+    _full_parity(w, synth.make_inputs(w, seed=31), B.DTYPE_FP32, TOL_FP32, flags)
+
+
+def test_gradients_accumulate_fp32():
+    w = synth.Workload("t", 203, 132, 268, 100, "fp32", "zipf")
+    inp = synth.make_inputs(w, seed=32)
+    st = runner.state_from_numpy(inp, B.DTYPE_FP32, w.V, flags=B.FLAG_ACCUM_GRADS)
+    start = {k: torch.randn_like(st.bufs[k]) for k in ("dW_gate", "dW_down")}
+    for k, v in start.items():
+        st.bufs[k].copy_(v)
+    st.step()
+    bw = O.backward(inp["dy"], inp["x"], inp["ids"], inp["W_gate"], inp["E"], inp["W_down"])
+    for k, v in start.items():
+        assert O.scaled_max_err(_np(st.bufs[k]), bw[k] + _np(v)) <= TOL_FP32, k
+
+
+def test_inputs_the_parts_cannot_carry():
+    """Infinities, NaN, values above bf16's range and below its smallest one: the same values are not
+    finite as in a chain of FMAs, and the others are as close to it as two fp32 sums are."""
+    T, d, F, V = 200, 128, 264, 50
+    out = []
+    for flags in (0, B.FLAG_SIMT):
+        w = synth.Workload("t", T, d, F, V, "fp32", "zipf")
+        st = runner.state_from_numpy(synth.make_inputs(w, seed=33), B.DTYPE_FP32, V, flags=flags, backward=False)
+        st.x[3, 5] = float("inf")
+        st.x[10, 7] = 3.4e38
+        st.x[11, 8] = float("nan")
+        st.W_gate[17, 9] = -float("inf")
+        st.x[50] *= 1e-30
+        st.x[51] *= 1e-37
+        st.x[52] = 0.0
+        st.dedup()
+        st.forward()
+        assert st.status() == B.OK
+        out.append(st.bufs["G"].double())
+    a, b = out
+    assert torch.equal(torch.isnan(a), torch.isnan(b))
+    inf = torch.isinf(a)
+    assert torch.equal(inf, torch.isinf(b)) and torch.equal(a[inf], b[inf])
+    ok = torch.isfinite(a)
+    assert ok[50].any() and ok[51].any()
+    for r in range(T):
+        m = ok[r]
+        if m.any():
+            scale = b[r][m].abs().max()
+            assert (a[r][m] - b[r][m]).abs().max() <= 4e-6 * scale, r      # sqrt(d) 2^-24 each, doubled
