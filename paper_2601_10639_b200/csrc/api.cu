@@ -310,9 +310,13 @@ int stem_ffn_forward(const stem_shape_t* shape, const void* x, const int32_t* id
     e = split_gemm(T, d, F, h3, false, wd3, false, kEpiStore, down, st);
     return e == cudaSuccess ? STEM_OK : cuda_fail(e);
   }
+  // a few rows: the weight matrices stream through once
+  const bool streams = use_tc(shape) && !(shape->flags & STEM_FLAG_SINGLE_CTA);
   {
     ProfScope prof("gate_gemm", st);
-    e = gemm(shape, T, F, d, x, false, W_gate, false, kEpiGate, gate, st);   // G = x W_gate^T, fused lookup
+    e = streams && stream_gemm_pays(T, F, d, kEpiGate)
+            ? launch_stream_gemm(T, F, d, x, W_gate, kEpiGate, gate, st)
+            : gemm(shape, T, F, d, x, false, W_gate, false, kEpiGate, gate, st);   // G = x W_gate^T, fused lookup
   }
   if (e != cudaSuccess) return cuda_fail(e);
   EpiParams down;
@@ -321,7 +325,9 @@ int stem_ffn_forward(const stem_shape_t* shape, const void* x, const int32_t* id
   down.sk_scratch = static_cast<char*>(ws) + w.sk_off; down.sk_bytes = w.sk_bytes;
   {
     ProfScope prof("down_gemm", st);
-    e = gemm(shape, T, d, F, H, false, W_down, false, kEpiStore, down, st);              // y = H W_down^T
+    e = streams && stream_gemm_pays(T, d, F, kEpiStore)
+            ? launch_stream_gemm(T, d, F, H, W_down, kEpiStore, down, st)
+            : gemm(shape, T, d, F, H, false, W_down, false, kEpiStore, down, st);        // y = H W_down^T
   }
   return e == cudaSuccess ? STEM_OK : cuda_fail(e);
 }

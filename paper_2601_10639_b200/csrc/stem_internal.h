@@ -120,6 +120,13 @@ cudaError_t launch_tc_gemm_token_pair(int K, int M1, int N1, const void* A1, con
 cudaError_t launch_tc_gemm_dagger(int M, int N, int K, const void* A, const void* B_gate, const void* B_up,
                                   const EpiParams& ep, cudaStream_t stream);
 
+// The weight-streaming form for batches of at most 256 rows (stream_gemm.cu):
+// C[t,f] = sum_k X[t,k] W[f,k], gate epilogue or plain bf16 store.  stream_gemm_pays: whether it
+// is the faster form for this size.
+cudaError_t launch_stream_gemm(int T, int F, int K, const void* X, const void* W, EpiKind kind, const EpiParams& ep,
+                               cudaStream_t stream);
+bool stream_gemm_pays(int T, int F, int K, EpiKind kind);
+
 size_t tc_gemm_scratch_bytes();
 void* tensor_map_encode_fn();   // cuTensorMapEncodeTiled, or NULL
 

@@ -1,0 +1,430 @@
+// bf16 contraction for batches of few rows (decode steps): the weight matrix streams through the tensor
+// cores once and the whole batch is the narrow operand.
+//
+//   C[t, f] = sum_k X(t, k) W(f, k)         X [T, K], W [F, K] row-major bf16, T <= 256
+//
+// The roles of the operands are swapped against the general kernel: 128 rows of W (256 for a CTA pair)
+// are the MMA's M, the batch padded to a multiple of 16 is its N.  A 256 x 256 tile of the general
+// kernel computes and stages 128 rows of batch per CTA whether they exist or not, and one row of such
+// tiles leaves most SMs without work.  Here the contraction is cut along k over the CTAs (pairs) of a
+// cluster until every SM streams an equal share of W; the CTAs leave their fp32 sums in shared memory,
+// and each adds one share of the batch over the cluster in ascending k and runs the epilogue on it,
+// pairs of neighbouring features per thread, so that table rows, G, H and y move in whole 128-byte lines.
+//
+// Bound: streaming W (3.6 TB/s from a cold memory with all SMs loading, and at most 70 - 98 GB/s into one
+// SM), on top of a chain of launch, first loads, last MMA, exchange and epilogue of some 5 us per kernel.
+// Measured, a forward pass (two of these kernels against two general ones), weights in L2 / not:
+//   d_model 2048, d_ff 8192   16 rows 32.4 -> 17.1 / 35.2 -> 20.8 us     128 rows 31.3 -> 26.0 us
+//   d_model 1024, d_ff 2816   16 rows 26.0 -> 12.1 us                    128 rows 27.0 -> 18.3 us
+// Loading W before the kernel that writes X has finished gained nothing: the two then share the memory's
+// bandwidth (23.7 us against 21.2 with it left out, 16 rows, weights not in L2).
+#include <cuda.h>
+
+#include "ptx_sm100.cuh"
+#include "stem_internal.h"
+
+namespace stem {
+namespace {
+
+constexpr int BM = 128;                 // rows of W per CTA
+constexpr int BK = 64;
+constexpr int kMaxT = 256;
+constexpr int kMaxStages = 12;
+constexpr int kEpiThreads = 256;
+constexpr int kThreads = 64 + kEpiThreads;
+constexpr long long kWaitLimitCycles = 2000000000ll;  // ~1 s at boost clock
+constexpr int kWBytes = BM * BK * 2;
+
+// bars: full[kMaxStages], empty[kMaxStages], done, drain; then tensor-memory address, abort flag, ids
+constexpr int kNumBars = 2 * kMaxStages + 2;
+constexpr int kTailBytes = kNumBars * 8 + 16 + kMaxT * 4;
+
+__device__ __forceinline__ float fast_sigmoid(float g) {   // as in the general kernel
+  float t;
+  asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(0.5f * g));
+  return fmaf(t, 0.5f, 0.5f);
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+template <int V> struct Int { static constexpr int value = V; };
+
+template <int KIND, int CTAS>
+__global__ void __launch_bounds__(kThreads)
+stream_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, int T, int F, int K,
+                   int n_pad, int stages, int ksplit, int tmem_cols, EpiParams ep) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = ptx::smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t* base_ptr = smem_raw + (base - raw);
+  const uint32_t x_bytes = static_cast<uint32_t>(n_pad / CTAS) * (BK * 2);
+  const uint32_t stage_bytes = kWBytes + x_bytes;
+  const uint32_t tail = max(stages * stage_bytes, static_cast<uint32_t>(n_pad) * BM * 4u);
+  const uint32_t bars = base + tail;
+  auto full_bar = [&](int s) { return bars + 8u * s; };
+  auto empty_bar = [&](int s) { return bars + 8u * (kMaxStages + s); };
+  const uint32_t done_bar = bars + 8u * (2 * kMaxStages), drain_bar = done_bar + 8u;
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(base_ptr + tail + kNumBars * 8);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + tail + kNumBars * 8 + 4);
+  int* s_ids = reinterpret_cast<int*>(base_ptr + tail + kNumBars * 8 + 16);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool clustered = CTAS * ksplit > 1;
+  const uint32_t crank = clustered ? ptx::cluster_ctarank() : 0u;
+  const uint32_t rank = CTAS == 2 ? crank & 1u : 0u, leader = crank - rank;
+  const int slice = static_cast<int>(crank) / CTAS;
+  const int f0 = (static_cast<int>(blockIdx.x) / (CTAS * ksplit) * CTAS + static_cast<int>(rank)) * BM;
+  const int k_blocks = (K + BK - 1) / BK;
+  const int kb0 = k_blocks * slice / ksplit, kb1 = k_blocks * (slice + 1) / ksplit;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < stages; ++s) { ptx::mbar_init(full_bar(s), 1); ptx::mbar_init(empty_bar(s), 1); }
+    ptx::mbar_init(done_bar, 1);
+    ptx::mbar_init(drain_bar, 1);
+    *abort_flag = 0;
+    ptx::fence_mbar_init();
+    ptx::prefetch_tensormap(&tmW);
+    ptx::prefetch_tensormap(&tmX);
+  }
+  if (warp == 1) {
+    if (CTAS == 2) {
+      ptx::tmem_alloc_pair(ptx::smem_u32(const_cast<uint32_t*>(tmem_slot)), tmem_cols);
+      ptx::tmem_relinquish_pair();
+    } else {
+      ptx::tmem_alloc(ptx::smem_u32(const_cast<uint32_t*>(tmem_slot)), tmem_cols);
+      ptx::tmem_relinquish();
+    }
+  }
+  ptx::tc_fence_before();
+  // a pair signals each other's barriers from here on; single CTAs meet only at the exchange of sums
+  if (CTAS == 2) ptx::cluster_sync(); else __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  int issued = 0;   // producer: k blocks handed to TMA so far
+  bool ok = true;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      auto load = [&](uint32_t dst, const CUtensorMap* map, int s, int k0, int row) {
+        if (CTAS == 2) ptx::tma_load_2d_pair(dst, map, ptx::mapa(full_bar(s), leader), k0, row);
+        else ptx::tma_load_2d(dst, map, full_bar(s), k0, row);
+      };
+      ptx::grid_dependency_wait();
+      ptx::grid_launch_dependents();
+      int s = 0; uint32_t ph = 0;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!ptx::mbar_wait_bounded(empty_bar(s), ph ^ 1u, abort_flag, kWaitLimitCycles)) {
+          report_error(ep.status, STEM_ERR_TIMEOUT, 1);
+          *abort_flag = 1; break;
+        }
+        if (rank == 0) ptx::mbar_arrive_expect_tx(full_bar(s), CTAS * stage_bytes);
+        load(base + s * stage_bytes, &tmW, s, kb * BK, f0);
+        load(base + s * stage_bytes + kWBytes, &tmX, s, kb * BK, rank * (n_pad / CTAS));
+        ++issued;
+        if (++s == stages) { s = 0; ph ^= 1u; }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0 && rank == 0) {
+      const uint32_t idesc = ptx::make_idesc_bf16(BM * CTAS, n_pad, false, false);
+      const uint16_t pair_mask = static_cast<uint16_t>(3u << leader);
+      int s = 0; uint32_t ph = 0;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (!ptx::mbar_wait_bounded(full_bar(s), ph, abort_flag, kWaitLimitCycles)) {
+          report_error(ep.status, STEM_ERR_TIMEOUT, 2);
+          *abort_flag = 1; ok = false; break;
+        }
+        ptx::tc_fence_after();
+        const uint32_t w_src = base + s * stage_bytes, x_src = w_src + kWBytes;
+#pragma unroll
+        for (int kk = 0; kk < BK / 16; ++kk) {
+          const uint64_t ad = ptx::make_smem_desc(w_src + kk * 32, 16, 1024), bd = ptx::make_smem_desc(x_src + kk * 32, 16, 1024);
+          if (CTAS == 2) ptx::mma_bf16_ss_pair(tmem_base, ad, bd, idesc, (kb > kb0 || kk > 0) ? 1u : 0u);
+          else ptx::mma_bf16_ss(tmem_base, ad, bd, idesc, (kb > kb0 || kk > 0) ? 1u : 0u);
+        }
+        if (CTAS == 2) ptx::mma_commit_pair(empty_bar(s), pair_mask); else ptx::mma_commit(empty_bar(s));
+        if (++s == stages) { s = 0; ph ^= 1u; }
+      }
+      if (ok) {
+        if (CTAS == 2) ptx::mma_commit_pair(done_bar, pair_mask); else ptx::mma_commit(done_bar);
+      } else {
+        // let MMAs already issued finish before TMEM is freed
+        if (CTAS == 2) ptx::mma_commit_pair(drain_bar, static_cast<uint16_t>(1u << leader)); else ptx::mma_commit(drain_bar);
+        int zero = 0;
+        ptx::mbar_wait_bounded(drain_bar, 0, &zero, kWaitLimitCycles);
+      }
+    }
+  } else {
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
+    const int et = threadIdx.x - 64;
+    // final stage: features f, f + 1 of the tokens first, first + step, ... of this CTA's share
+    const int f = f0 + (et & 63) * 2, first = slice + ksplit * (et >> 6), step = ksplit * (kEpiThreads / 64);
+    const bool f_ok = f < F;
+    // Sixteen 8-byte reads of other CTAs' sums are in flight per thread: those of 8 tokens from 2 CTAs, or
+    // of 4 tokens from 4 CTAs at a time.
+    const int batch = ksplit <= 2 ? 8 : 4;
+    uint32_t e[8];
+    auto request = [&](int t0) {      // table-row pairs of the next tokens
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int t = t0 + i * step;
+        if (KIND == kEpiGate && f_ok && i < batch && t < T)
+          e[i] = __ldg(reinterpret_cast<const uint32_t*>(static_cast<const __nv_bfloat16*>(ep.E) + static_cast<size_t>(s_ids[t]) * F + f));
+      }
+    };
+    if (KIND == kEpiGate) {
+      if (et < T) {
+        int id = ep.ids != nullptr ? ep.ids[et] : et;
+        if (id < 0 || id >= ep.V) {
+          report_error(ep.status, STEM_ERR_ID_RANGE, et);
+          id = id < 0 ? 0 : ep.V - 1;
+        }
+        s_ids[et] = id;
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
+      request(first);
+    }
+    bool mine = ptx::mbar_wait_bounded(done_bar, 0, abort_flag, kWaitLimitCycles);
+    mine = __all_sync(0xffffffffu, mine);
+    if (!mine) {
+      if (lane == 0) { report_error(ep.status, STEM_ERR_TIMEOUT, 4); *abort_flag = 1; }
+      ok = false;
+    } else {
+      // Every copy of this CTA has landed and every MMA on it is complete: the operand ring is free for
+      // the sums, token by token (128 features of a token side by side).
+      ptx::tc_fence_after();
+      const int q = warp & 3, half = (warp - 2) >> 2;
+      float* part = reinterpret_cast<float*>(base_ptr) + q * 32 + lane;
+      for (int c = half * 16; c < n_pad; c += 32) {
+        uint32_t v[16];
+        ptx::tmem_ld_32x16(tmem_base + c + (static_cast<uint32_t>(q * 32) << 16), v);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) part[(c + i) * BM] = __uint_as_float(v[i]);
+      }
+      ptx::tc_fence_before();
+    }
+    __syncwarp();
+    // Every epilogue thread of the cluster meets here, also after a timeout (the other warps: below).
+    if (clustered) ptx::cluster_sync(); else asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
+    if (ok && f_ok) {
+      const uint32_t sums = base + 8u * (et & 63);
+      // (Rolled up on purpose: this runs once, and a body unrolled over the tokens took 8300 cycles to fetch.)
+      auto finish = [&](auto tokens, auto ctas) {
+        constexpr int TB = decltype(tokens)::value, KB = decltype(ctas)::value;
+#pragma unroll 1
+        for (int t0 = first; t0 < T; t0 += TB * step) {
+          uint32_t cur[TB];
+          float a0[TB], a1[TB];
+#pragma unroll
+          for (int i = 0; i < TB; ++i) { cur[i] = e[i]; a0[i] = 0.0f; a1[i] = 0.0f; }
+          if (t0 + TB * step < T) request(t0 + TB * step);
+#pragma unroll 1
+          for (int k0 = 0; k0 < ksplit; k0 += KB) {
+            float p0[KB][TB], p1[KB][TB];
+#pragma unroll
+            for (int k = 0; k < KB; ++k) {
+              const uint32_t src = sums + 4u * BM * t0;
+              const uint32_t at = clustered ? ptx::mapa(src, min(k0 + k, ksplit - 1) * CTAS + rank) : src;
+#pragma unroll
+              for (int i = 0; i < TB; ++i) {
+                p0[k][i] = p1[k][i] = 0.0f;
+                if (k0 + k < ksplit && t0 + i * step < T) ptx::ld_shared_cluster_f32x2(at + 4u * BM * i * step, p0[k][i], p1[k][i]);
+              }
+            }
+#pragma unroll
+            for (int k = 0; k < KB; ++k)
+#pragma unroll
+              for (int i = 0; i < TB; ++i) { a0[i] += p0[k][i]; a1[i] += p1[k][i]; }
+          }
+#pragma unroll
+          for (int i = 0; i < TB; ++i) {
+            const int t = t0 + i * step;
+            if (t < T) {
+              const size_t o = static_cast<size_t>(t) * F + f;
+              if (KIND == kEpiGate) {
+                const float u0 = __uint_as_float(cur[i] << 16), u1 = __uint_as_float(cur[i] & 0xFFFF0000u);
+                *reinterpret_cast<uint32_t*>(static_cast<__nv_bfloat16*>(ep.H) + o) =
+                    pack_bf16(a0[i] * fast_sigmoid(a0[i]) * u0, a1[i] * fast_sigmoid(a1[i]) * u1);
+                if (ep.G) *reinterpret_cast<uint32_t*>(static_cast<__nv_bfloat16*>(ep.G) + o) = pack_bf16(a0[i], a1[i]);
+              } else {
+                *reinterpret_cast<uint32_t*>(static_cast<__nv_bfloat16*>(ep.out) + o) = pack_bf16(a0[i], a1[i]);
+              }
+            }
+          }
+        }
+      };
+      if (batch == 8) finish(Int<8>{}, Int<2>{}); else finish(Int<4>{}, Int<4>{});
+    }
+    __syncwarp();
+  }
+
+  if (clustered && warp < 2) { __syncwarp(); ptx::cluster_sync(); }   // (the epilogue warps': above)
+  __syncthreads();
+  if (*abort_flag != 0 && threadIdx.x == 0) {
+    // wait (bounded) for copies still in flight; the second CTA of a pair cannot poll the barriers
+    // its bytes are counted on and waits out a fixed interval (far longer than a copy takes)
+    int zero = 0;
+    if (rank == 0) {
+      for (int j = issued > stages ? issued - stages : 0; j < issued; ++j)
+        ptx::mbar_wait_bounded(full_bar(j % stages), (j / stages) & 1, &zero, kWaitLimitCycles / 16);
+    } else {
+      const long long t0 = clock64();
+      while (clock64() - t0 < 2000000ll) { }
+    }
+  }
+  // No CTA of a cluster leaves (or frees TMEM) while another can still signal its barriers, read its
+  // shared memory or write its accumulators.
+  if (clustered) ptx::cluster_sync(); else __syncthreads();
+  if (warp == 1) {
+    ptx::tc_fence_after();
+    if (CTAS == 2) ptx::tmem_dealloc_pair(tmem_base, tmem_cols); else ptx::tmem_dealloc(tmem_base, tmem_cols);
+  }
+}
+
+// Row-major bf16 [rows, cols]; box = 64 columns x box_rows rows, 128-byte swizzle.
+bool encode_operand(CUtensorMap* map, const void* ptr, int rows, int cols, int box_rows) {
+  const auto fn = reinterpret_cast<CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                                const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
+                                                CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
+                                                CUtensorMapFloatOOBfill)>(tensor_map_encode_fn());
+  if (!fn) return false;
+  const cuuint64_t dims[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
+  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(cols) * 2};
+  const cuuint32_t box[2] = {64u, static_cast<cuuint32_t>(box_rows)};
+  const cuuint32_t estr[2] = {1u, 1u};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Shared memory of a CTA: batches of up to 128 rows leave room for a second CTA on the SM.  (With all of it
+// a forward pass of 128 rows took 38.8 us against 33.3: two rounds of clusters of 8.)
+constexpr int kMaxSmem = 232448;
+int smem_budget(int n_pad) { return n_pad <= 128 ? 113 * 1024 : kMaxSmem; }
+
+// Clusters of `size` CTAs that run at once with one CTA per SM (an SM left over in a GPC is no help to a
+// cluster that needs more of them: 15 clusters of 8, not 18).  Asked once per device and size.
+int max_clusters(int size) {
+  static int cached[64][9] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return device_sm_count() / size;
+  if (cached[dev][size] == 0) {
+    int n = 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(device_sm_count() / size * size));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kMaxSmem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(size);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    auto kern = stream_gemm_kernel<kEpiStore, 1>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+      cudaGetLastError();
+      n = device_sm_count() / size;
+    }
+    cached[dev][size] = n;
+  }
+  return cached[dev][size];
+}
+
+// Single CTAs or pairs, and CTAs along k.  What a CTA must load sets the pace: its k range times 128 rows
+// of W and its rows of X (half of the batch in a pair), times the rounds its clusters take.  Narrow
+// batches get no more CTAs than there are SMs, though two fit one: the second place is a cluster's that
+// finds its GPC full (twice the CTAs at half the k range measured the same at 16 rows and 10 % slower at 128).
+// (The MMA's N is a multiple of 16, in a pair of 32.)
+struct Plan { int ctas, ksplit, n_pad; long long rows; };
+Plan make_plan(int T, int F, int K) {
+  const int k_blocks = (K + BK - 1) / BK, slots = device_sm_count();
+  Plan best{1, 1, 0, 0};
+  for (int ctas = 1; ctas <= 2; ++ctas) {
+    const int tiles = (F + BM * ctas - 1) / (BM * ctas), n_pad = (T + 16 * ctas - 1) / (16 * ctas) * (16 * ctas);
+    for (int sp = 1; sp * ctas <= 8; ++sp) {
+      if (sp > 1 && (k_blocks < 2 * sp || static_cast<long long>(tiles) * ctas * sp > slots)) break;
+      const int at_once = n_pad <= 128 ? slots / (ctas * sp) : max_clusters(ctas * sp);
+      const long long rounds = (tiles + at_once - 1) / at_once;
+      const long long rows = rounds * ((k_blocks + sp - 1) / sp) * (BM + n_pad / ctas);
+      if (best.rows == 0 || rows < best.rows) best = {ctas, sp, n_pad, rows};
+    }
+  }
+  return best;
+}
+
+template <int KIND, int CTAS>
+cudaError_t launch_inst(const void* X, const void* W, int T, int F, int K, const Plan& pl, const EpiParams& ep,
+                        cudaStream_t stream) {
+  const int n_pad = pl.n_pad, ksplit = pl.ksplit;
+  auto kern = stream_gemm_kernel<KIND, CTAS>;
+  static PerDeviceOnce configured;
+  if (cudaError_t ce = configured.run([&] {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+      }))
+    return ce;
+  CUtensorMap tmW, tmX;
+  if (!encode_operand(&tmW, W, F, K, BM) || !encode_operand(&tmX, X, T, K, n_pad / CTAS)) return cudaErrorNotSupported;
+  const int k_blocks = (K + BK - 1) / BK, my_blocks = (k_blocks + ksplit - 1) / ksplit;
+  const int stage_bytes = kWBytes + n_pad / CTAS * BK * 2;
+  const int budget = smem_budget(n_pad) - kTailBytes - 1024;
+  int stages = budget / stage_bytes;
+  if (stages > kMaxStages) stages = kMaxStages;
+  if (stages > my_blocks) stages = my_blocks;
+  int ring = stages * stage_bytes;
+  if (ring < n_pad * BM * 4) ring = n_pad * BM * 4;    // the sums take the ring's place
+  int tmem_cols = 32;
+  while (tmem_cols < n_pad) tmem_cols *= 2;
+  const int tiles = (F + BM * CTAS - 1) / (BM * CTAS);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(tiles * CTAS * ksplit));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = ring + kTailBytes + 1024;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned>(CTAS * ksplit);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = CTAS * ksplit > 1 ? 2 : 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmW, tmX, T, F, K, n_pad, stages, ksplit, tmem_cols, ep);
+  count_launches(1);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_stream_gemm(int T, int F, int K, const void* X, const void* W, EpiKind kind, const EpiParams& ep,
+                               cudaStream_t stream) {
+  if (T <= 0 || F <= 0) return cudaSuccess;
+  if (T > kMaxT || K <= 0 || (F % 8) || (K % 8) || (kind != kEpiGate && kind != kEpiStore) ||
+      (kind == kEpiStore && (ep.out_fp32 || ep.accumulate)))
+    return cudaErrorNotSupported;
+  const Plan pl = make_plan(T, F, K);
+  if (kind == kEpiGate) {
+    if (pl.ctas == 2) return launch_inst<kEpiGate, 2>(X, W, T, F, K, pl, ep, stream);
+    return launch_inst<kEpiGate, 1>(X, W, T, F, K, pl, ep, stream);
+  }
+  if (pl.ctas == 2) return launch_inst<kEpiStore, 2>(X, W, T, F, K, pl, ep, stream);
+  return launch_inst<kEpiStore, 1>(X, W, T, F, K, pl, ep, stream);
+}
+
+// Above 128 rows a CTA has no room for a second one beside it, and the exchange (fp32 sums of the whole batch)
+// outweighs what is saved, but for a plain store of a short k range per CTA.  Measured, general kernel against
+// this one: gate, 144 rows: 20.4 / 22.6 us at 2048 x 8192, 14.4 / 16.4 at 1024 x 2816; down, 256 rows: 22.6 /
+// 18.4 us at 1024 x 2816 (6 blocks x 384 rows), 21.5 / 22.5 at 1536 x 5000 (10 x 384), 23.5 / 24.7 at 2048 x 8192.
+bool stream_gemm_pays(int T, int F, int K, EpiKind kind) {
+  if (T <= 128) return true;
+  return kind == kEpiStore && T <= kMaxT && make_plan(T, F, K).rows <= 3000;
+}
+
+}  // namespace stem
