@@ -27,28 +27,8 @@ __host__ __device__ inline Split make_split(int T) {
   return {n_ctas, epw};
 }
 
-// The kernels of one dedup call are launched with programmatic stream serialisation: each
-// may be scheduled while its predecessor is still draining, waits here for the predecessor's
-// results to be complete and visible, and then lets its own successor be scheduled.  That
-// takes most of the launch gaps out of a chain of six few-microsecond kernels.
-__device__ __forceinline__ void pdl_wait_then_release() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-template <typename... KArgs, typename... Args>
-cudaError_t launch_chained(void (*kernel)(KArgs...), int grid, int block, cudaStream_t stream, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(grid));
-  cfg.blockDim = dim3(static_cast<unsigned>(block));
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
+// The kernels of one dedup call are launched with programmatic stream serialisation (launch_chained).
+// That takes most of the launch gaps out of a chain of six few-microsecond kernels.
 
 __device__ __forceinline__ int clamp_id(int key, int V) { return key < 0 ? 0 : (key >= V ? V - 1 : key); }
 
@@ -240,6 +220,7 @@ dedup_small_kernel(int T, int V, const int32_t* __restrict__ ids, int32_t* __res
   __shared__ int s_sorted[kCtaThreads];
   __shared__ int s_perm[kCtaThreads];
   __shared__ int s_warp[kWarps];
+  pdl_wait_then_release();
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   int id = 0x7fffffff;
   if (t < T) {
@@ -354,10 +335,10 @@ cudaError_t launch_dedup(int T, int V, const int32_t* ids, int32_t* unique_ids, 
     return cudaGetLastError();
   }
   if (T <= kCtaThreads) {
-    dedup_small_kernel<<<1, kCtaThreads, 0, stream>>>(T, V, ids, unique_ids, n_unique, inverse, perm, seg_offsets,
-                                                    status);
+    cudaError_t e = launch_chained(dedup_small_kernel, 1, kCtaThreads, stream, T, V, ids, unique_ids, n_unique, inverse,
+                                   perm, seg_offsets, status);
     count_launches(1);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
   }
   const Split sp = make_split(T);
   const size_t tb = align_up(static_cast<size_t>(T) * 4, 256);

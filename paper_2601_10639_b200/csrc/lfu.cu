@@ -25,6 +25,7 @@ constexpr int kKeyMax = 0x7ffffffe;
 __global__ void __launch_bounds__(kThreads)
 lfu_touch_kernel(int n, int V, const int32_t* __restrict__ ids, int32_t* freq,
                  const int32_t* __restrict__ hot_slot, int32_t* stats, int32_t* status) {
+  pdl_wait_then_release();
   int hits = 0, misses = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     int id = ids[i];
@@ -134,9 +135,9 @@ cudaError_t launch_lfu_touch(int n, int V, const int32_t* ids, int32_t* freq, co
                              int32_t* stats, int32_t* status, cudaStream_t stream) {
   if (n <= 0) return cudaSuccess;
   const int blocks = (n + kThreads - 1) / kThreads < 64 ? (n + kThreads - 1) / kThreads : 64;
-  lfu_touch_kernel<<<blocks, kThreads, 0, stream>>>(n, V, ids, freq, hot_slot, stats, status);
+  cudaError_t e = launch_chained(lfu_touch_kernel, blocks, kThreads, stream, n, V, ids, freq, hot_slot, stats, status);
   count_launches(1);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_lfu_refresh(int V, int K, size_t row_bytes, const int32_t* freq, int32_t* hot_slot,

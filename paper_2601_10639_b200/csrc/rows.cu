@@ -17,12 +17,16 @@ namespace {
 constexpr int kThreads = 256;          // device-to-device gathers
 constexpr int kHostLinkCtas = 32;
 constexpr int kHostLinkThreads = 128;
+// A decode step's rows are few and the step waits for them: one CTA per row, so that no row's chain of
+// id, slot, host read waits for another's.  (With 32 CTAs such chains were five rows long at 147 rows.)
+constexpr int kDecodeRows = 512;
 
 __global__ void __launch_bounds__(kThreads)
 gather_rows_kernel(int max_rows, int V, int vec_per_row, const int32_t* __restrict__ ids,
                    const int32_t* __restrict__ n_ids, const uint4* __restrict__ table,
                    const uint4* __restrict__ hot_rows, const int32_t* __restrict__ hot_slot,
                    uint4* __restrict__ dst, int32_t* status, int32_t* stats) {
+  pdl_wait_then_release();
   // the count is a device scalar the host never saw: never trust it beyond the buffers' capacity
   int n = *n_ids;
   if (n > max_rows || n < 0) {
@@ -94,6 +98,7 @@ gather_rows_flat_kernel(int max_rows, int V, int vec_per_row, const int32_t* __r
                         const int32_t* __restrict__ n_ids, const uint4* __restrict__ table,
                         const uint4* __restrict__ hot_rows, const int32_t* __restrict__ hot_slot,
                         uint4* __restrict__ dst, int32_t* status, int32_t* stats) {
+  pdl_wait_then_release();
   int n = *n_ids;
   if (n > max_rows || n < 0) {
     if (blockIdx.x == 0 && threadIdx.x == 0) report_error(status, STEM_ERR_COUNT_RANGE, n);
@@ -169,26 +174,26 @@ cudaError_t launch_gather_rows(int max_rows, int V, size_t row_bytes, const int3
   const int lanes_per_row = vec < threads ? vec : threads;
   const int rows_per_cta = threads / lanes_per_row;
   int blocks = (max_rows + rows_per_cta - 1) / rows_per_cta;
-  const int cap = table_on_host ? kHostLinkCtas : device_sm_count() * 8;
+  const int cap = max_rows <= kDecodeRows ? kDecodeRows : kHostLinkCtas;
   if (blocks > cap) blocks = cap;
   if (!table_on_host) {
     // a device table: flat copy, as many CTAs as the largest possible count needs, up to 8 per SM
     const size_t per_cta = static_cast<size_t>(kThreads) * kFlatBatch;
     const size_t need = (static_cast<size_t>(max_rows) * vec + per_cta - 1) / per_cta;
     const int grid = static_cast<int>(need < static_cast<size_t>(device_sm_count()) * 8 ? need : device_sm_count() * 8);
-    gather_rows_flat_kernel<<<grid > 0 ? grid : 1, kThreads, 0, stream>>>(
-        max_rows, V, vec, ids, n_ids, static_cast<const uint4*>(table), static_cast<const uint4*>(hot_rows), hot_slot,
-        static_cast<uint4*>(dst), status, stats);
+    cudaError_t e = launch_chained(gather_rows_flat_kernel, grid > 0 ? grid : 1, kThreads, stream, max_rows, V, vec, ids,
+                                   n_ids, static_cast<const uint4*>(table), static_cast<const uint4*>(hot_rows), hot_slot,
+                                   static_cast<uint4*>(dst), status, stats);
     count_launches(1);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
   }
   static PerDeviceOnce configured;
   if (cudaError_t ce = configured.run([] { return prefer_max_shared(gather_rows_kernel); })) return ce;
-  gather_rows_kernel<<<blocks, threads, 0, stream>>>(max_rows, V, vec, ids, n_ids, static_cast<const uint4*>(table),
-                                                    static_cast<const uint4*>(hot_rows), hot_slot,
-                                                    static_cast<uint4*>(dst), status, stats);
+  cudaError_t e = launch_chained(gather_rows_kernel, blocks, threads, stream, max_rows, V, vec, ids, n_ids,
+                                 static_cast<const uint4*>(table), static_cast<const uint4*>(hot_rows), hot_slot,
+                                 static_cast<uint4*>(dst), status, stats);
   count_launches(1);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_writeback_rows(int max_rows, size_t row_bytes, const void* rows,

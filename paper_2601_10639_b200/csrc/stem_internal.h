@@ -197,4 +197,26 @@ struct PerDeviceOnce {
 };
 void count_launches(int n);  // bookkeeping for stem_launch_count()
 
+// Launch with programmatic stream serialisation: the kernel may be scheduled while its predecessor in
+// the stream is still draining.  It must wait for the predecessor (griddepcontrol.wait) before it
+// touches anything an earlier kernel wrote or still reads, and should then let its own successor be
+// scheduled (griddepcontrol.launch_dependents).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_chained(void (*kernel)(KArgs...), int grid, int block, cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(grid));
+  cfg.blockDim = dim3(static_cast<unsigned>(block));
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+__device__ __forceinline__ void pdl_wait_then_release() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 }  // namespace stem
