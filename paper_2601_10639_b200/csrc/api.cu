@@ -403,8 +403,8 @@ int stem_ffn_backward(const stem_shape_t* shape, const void* dy, const void* x, 
     // contract over the tokens, and their output tiles together fill the SMs (at the 350M shape
     // each has 44 tiles for 74 CTA pairs) with one split tail and one fix-up instead of two
     ProfScope prof("dw_pair_gemm", st);
-    e = launch_tc_gemm_token_pair(T, d, F, dy, H_save, dW_down, F, d, dG, x, dW_gate, gp,
-                                  !(shape->flags & STEM_FLAG_SINGLE_CTA), st);
+    e = launch_tc_gemm_token_pair(T, d, F, dy, H_save, dW_down, F, d, dG, x, dW_gate, nullptr, nullptr,
+                                  gp, !(shape->flags & STEM_FLAG_SINGLE_CTA), st);
     if (e != cudaSuccess) return cuda_fail(e);
   } else {
     if (dW_down) {  // dW_down[i,j] = sum_t dy[t,i] H[t,j]
@@ -621,8 +621,9 @@ int stem_dagger_backward(const stem_shape_t* shape, const void* dy, const void* 
     ProfScope prof(name, st);
     return gemm(shape, M, N, T, A, true, Bm, true, kEpiStore, p, st);   // contraction over the tokens
   };
-  if (dW_down && (e = split ? split_grad("dw_down_gemm", dW_down, d, F, dy3, h3)
-                            : grad("dw_down_gemm", dW_down, d, F, dy, H_save)) != cudaSuccess) return cuda_fail(e);
+  const bool together = use_tc(shape) && dW_down && dW_gate && dW_up;   // one launch for the three weight gradients
+  if (!together && dW_down && (e = split ? split_grad("dw_down_gemm", dW_down, d, F, dy3, h3)
+                                         : grad("dw_down_gemm", dW_down, d, F, dy, H_save)) != cudaSuccess) return cuda_fail(e);
   if (dE_rows) {
     ProfScope prof("seg_reduce", st);
     e = launch_segreduce(T, F, shape->dtype, shape->grad_dtype, dU, perm, seg_offsets, n_unique, dE_rows,
@@ -630,11 +631,27 @@ int stem_dagger_backward(const stem_shape_t* shape, const void* dy, const void* 
     if (e != cudaSuccess) return cuda_fail(e);
   }
   if (split && (dW_up || dx) && (e = split3({du3, wu3}, st)) != cudaSuccess) return cuda_fail(e);
-  if (dW_gate && (e = split ? split_grad("dw_gate_gemm", dW_gate, F, d, dg3, x3)
-                            : grad("dw_gate_gemm", dW_gate, F, d, dG, x)) != cudaSuccess) return cuda_fail(e);
-  if (dW_up && (e = split ? split_grad("dw_up_gemm", dW_up, F, d, du3, x3)
-                          : grad("dw_up_gemm", dW_up, F, d, dU, x)) != cudaSuccess) return cuda_fail(e);
-  if (dx) {  // dx = dG W_gate + dU W_up: the second product is added onto the first in its epilogue
+  if (together) {
+    EpiParams p; p.out_fp32 = grad_fp32; p.status = status_of(ws);
+    p.accumulate = (shape->flags & STEM_FLAG_ACCUM_GRADS) != 0;
+    p.sk_scratch = base + w.sk_off; p.sk_bytes = w.sk_bytes;
+    ProfScope prof("dw_triple_gemm", st);
+    e = launch_tc_gemm_token_pair(T, d, F, dy, H_save, dW_down, F, d, dG, x, dW_gate, dU, dW_up, p,
+                                  !(shape->flags & STEM_FLAG_SINGLE_CTA), st);
+    if (e != cudaSuccess) return cuda_fail(e);
+  } else {
+    if (dW_gate && (e = split ? split_grad("dw_gate_gemm", dW_gate, F, d, dg3, x3)
+                              : grad("dw_gate_gemm", dW_gate, F, d, dG, x)) != cudaSuccess) return cuda_fail(e);
+    if (dW_up && (e = split ? split_grad("dw_up_gemm", dW_up, F, d, du3, x3)
+                            : grad("dw_up_gemm", dW_up, F, d, dU, x)) != cudaSuccess) return cuda_fail(e);
+  }
+  if (dx && use_tc(shape)) {  // dx = dG W_gate + dU W_up, one contraction over both
+    EpiParams p; p.out = dx; p.status = status_of(ws);
+    p.sk_scratch = base + w.sk_off; p.sk_bytes = w.sk_bytes;
+    ProfScope prof("dx_gemm", st);
+    e = launch_tc_gemm_sum(T, d, F, dG, W_gate, dU, W_up, p, !(shape->flags & STEM_FLAG_SINGLE_CTA), st);
+    if (e != cudaSuccess) return cuda_fail(e);
+  } else if (dx) {  // the second product is added onto the first in its epilogue
     EpiParams p; p.out = dx; p.out_fp32 = shape->dtype == STEM_DTYPE_FP32; p.status = status_of(ws);
     {
       ProfScope prof("dx_gemm", st);

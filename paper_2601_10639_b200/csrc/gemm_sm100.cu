@@ -241,8 +241,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmC0, const __grid_constant__ CUtensorMap tmC1,
                const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
-               const __grid_constant__ CUtensorMap tmC2,
-               int M, int N, int K, int M2, int N2, int group_m, int dp_tiles, int split, EpiParams ep) {
+               const __grid_constant__ CUtensorMap tmC2, const __grid_constant__ CUtensorMap tmA3,
+               const __grid_constant__ CUtensorMap tmC3, int M, int N, int K, int M2, int N2, int third, int k_switch,
+               int group_m, int dp_tiles, int split, EpiParams ep) {
   constexpr bool kDual = KIND == kEpiDagger;      // two products (gate, up) of every A tile
   using L = Smem<BN, STAGES, CTAS, kDual>;
   constexpr int kAccCols = kDual ? 2 * BN : BN;   // TMEM columns of one accumulator set
@@ -269,8 +270,17 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   // fill the machine together where each alone would leave SMs idle.
   const int tiles_m2 = KIND == kEpiStore && M2 > 0 ? (M2 + BM * CTAS - 1) / (BM * CTAS) : 0;
   const int tiles_n2 = KIND == kEpiStore && M2 > 0 ? (N2 + BN - 1) / BN : 0;
-  const int num_tiles1 = tiles_m * tiles_n;
-  const int num_tiles = num_tiles1 + tiles_m2 * tiles_n2;
+  // A third one (third != 0) has the second's B and extents, with an A and an output of its own.
+  const int num_tiles1 = tiles_m * tiles_n, num_tiles2 = tiles_m2 * tiles_n2;
+  const int num_tiles = num_tiles1 + num_tiles2 * (third ? 2 : 1);
+  // product of the launch that a tile belongs to (0, 1, 2), and the tile's coordinates in it
+  auto product_of = [&](int tile) {
+    return KIND == kEpiStore && tile >= num_tiles1 ? (tile >= num_tiles1 + num_tiles2 ? 2 : 1) : 0;
+  };
+  auto coord_of = [&](int tile, int product) {
+    return product > 0 ? tile_coord(tile - num_tiles1 - (product - 1) * num_tiles2, tiles_m2, tiles_n2, group_m)
+                       : tile_coord(tile, tiles_m, tiles_n, group_m);
+  };
   const int k_blocks = (K + BK - 1) / BK;
   constexpr uint32_t kTmemCols = 2 * kAccCols;
   static_assert(kTmemCols <= 512, "two accumulator sets must fit the 512 TMEM columns");
@@ -287,6 +297,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     ptx::prefetch_tensormap(&tmC0);
     if (KIND == kEpiGate || KIND == kEpiDH || kDual) ptx::prefetch_tensormap(&tmC1);
     if (kDual) { ptx::prefetch_tensormap(&tmB2); ptx::prefetch_tensormap(&tmC2); }
+    if (KIND == kEpiStore && k_switch < k_blocks) { ptx::prefetch_tensormap(&tmA2); ptx::prefetch_tensormap(&tmB2); }
+    if (KIND == kEpiStore && third) { ptx::prefetch_tensormap(&tmA3); ptx::prefetch_tensormap(&tmC3); }
     if (KIND == kEpiStore && M2 > 0) {
       ptx::prefetch_tensormap(&tmA2);
       ptx::prefetch_tensormap(&tmB2);
@@ -320,11 +332,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       bool ok = true;
       Work w;
       for (int i = 0; ok && work.get(i, w); ++i) {
-        const bool second = KIND == kEpiStore && w.tile >= num_tiles1;
-        const TileCoord tc = second ? tile_coord(w.tile - num_tiles1, tiles_m2, tiles_n2, group_m)
-                                    : tile_coord(w.tile, tiles_m, tiles_n, group_m);
-        const CUtensorMap* mapA = second ? &tmA2 : &tmA;
-        const CUtensorMap* mapB = second ? &tmB2 : &tmB;
+        const int product = product_of(w.tile);
+        const TileCoord tc = coord_of(w.tile, product);
+        const CUtensorMap* mapA = product == 0 ? &tmA : (product == 1 ? &tmA2 : &tmA3);
+        const CUtensorMap* mapB = product == 0 ? &tmB : &tmB2;
         // this CTA's rows of A and its share of the columns of B
         const int m0 = (tc.m_blk * CTAS + rank) * BM, n0 = tc.n_blk * BN + rank * (BN / CTAS);
         for (int kb = w.kb0; kb < w.kb1; ++kb) {
@@ -340,7 +351,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           auto load = [&](uint32_t dst, const CUtensorMap* map, int c0, int c1) {
             if (CTAS == 2) ptx::tma_load_2d_pair(dst, map, fb, c0, c1); else ptx::tma_load_2d(dst, map, fb, c0, c1);
           };
-          const int k0 = kb * BK;
+          int k0 = kb * BK;
+          if (KIND == kEpiStore && kb >= k_switch) {   // the contraction goes on over a second pair of operands
+            mapA = &tmA2;
+            mapB = &tmB2;
+            k0 -= k_switch * BK;
+          }
           if (A_MN) {
 #pragma unroll
             for (int j = 0; j < BM / 64; ++j) load(a_dst + j * kAtomBytes, mapA, m0 + 64 * j, k0);
@@ -430,11 +446,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     bool ok = true;
     Work w;
     for (int i = 0; ok && work.get(i, w); ++i) {
-      const bool second = KIND == kEpiStore && w.tile >= num_tiles1;
-      const TileCoord tc = second ? tile_coord(w.tile - num_tiles1, tiles_m2, tiles_n2, group_m)
-                                  : tile_coord(w.tile, tiles_m, tiles_n, group_m);
-      const CUtensorMap* mapC = second ? &tmC2 : &tmC0;
-      const int M_ = second ? M2 : M, N_ = second ? N2 : N;    // extents of the product this tile belongs to
+      const int product = product_of(w.tile);
+      const TileCoord tc = coord_of(w.tile, product);
+      const CUtensorMap* mapC = product == 0 ? &tmC0 : (product == 1 ? &tmC2 : &tmC3);
+      const int M_ = product > 0 ? M2 : M, N_ = product > 0 ? N2 : N;    // extents of the product this tile belongs to
       const int m_warp = (tc.m_blk * CTAS + rank) * BM + q * 32;  // first row of this warp's 32-row block
       const int m = m_warp + lane;
       const int n0 = tc.n_blk * BN + half * (BN / 2);
@@ -558,17 +573,18 @@ template <int BN, int CTAS>
 __global__ void __launch_bounds__(256)
 tail_fixup_kernel(int M, int N, int dp_tiles, int tail, int split, int tiles_m, int tiles_n, int group_m,
                   const float* __restrict__ partial, void* __restrict__ out, int out_fp32, int accumulate,
-                  int M2, int N2, int tiles_m2, int tiles_n2, void* __restrict__ out2) {
+                  int M2, int N2, int tiles_m2, int tiles_n2, void* __restrict__ out2, void* __restrict__ out3) {
   constexpr int TM = BM * CTAS;
   ptx::grid_dependency_wait();
   ptx::grid_launch_dependents();
   const int j = blockIdx.x;
-  // tiles of a second product riding in the same launch are numbered after the first product's
-  const int num_tiles1 = tiles_m * tiles_n;
-  const bool second = dp_tiles + j >= num_tiles1;
-  const TileCoord tc = second ? tile_coord(dp_tiles + j - num_tiles1, tiles_m2, tiles_n2, group_m)
+  // tiles of a second (and third) product riding in the same launch are numbered after the first product's
+  const int num_tiles1 = tiles_m * tiles_n, num_tiles2 = tiles_m2 * tiles_n2;
+  const int in_second = dp_tiles + j - num_tiles1;
+  const bool second = in_second >= 0, third = second && in_second >= num_tiles2;
+  const TileCoord tc = second ? tile_coord(in_second - (third ? num_tiles2 : 0), tiles_m2, tiles_n2, group_m)
                               : tile_coord(dp_tiles + j, tiles_m, tiles_n, group_m);
-  if (second) { M = M2; N = N2; out = out2; }
+  if (second) { M = M2; N = N2; out = third ? out3 : out2; }
   const int r0 = blockIdx.y * kFixRows;
   for (int e = threadIdx.x; e < kFixRows * (BN / 4); e += 256) {
     const int r = r0 + e / (BN / 4), c = (e % (BN / 4)) * 4;
@@ -643,11 +659,18 @@ bool encode_out_map(CUtensorMap* map, const void* ptr, int rows, int cols, bool 
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// A second product C2 = A2 B2^T with the same contraction length and operand layouts, carried by
-// the same launch (plain stores only); M == 0 means none.
-// The same parameter slots carry the second B operand (B) and the third output (C) of the
-// two-product kind kEpiDagger, with M == 0 and `maps` set.
-struct SecondMaps { CUtensorMap A, B, C; int M = 0, N = 0; void* out = nullptr; bool maps = false; };
+// What else the launch carries (plain stores, and the two-product kind kEpiDagger).
+//   M > 0       a second product C2 = A2 B2^T with the same contraction length and operand layouts;
+//               out3 != NULL: a third one, C3 = A3 B2^T, with the second's extents
+//   k_switch    from this k block on the operands are A2, B2: C = A B^T + A2 B2^T
+//   maps        kEpiDagger: B is the second B operand and C the third output
+struct SecondMaps {
+  CUtensorMap A, B, C, A3, C3;
+  int M = 0, N = 0, k_switch = 0x7fffffff;
+  void* out = nullptr;
+  void* out3 = nullptr;
+  bool maps = false;
+};
 
 template <bool A_MN, bool B_MN, int KIND, int BN, int STAGES, bool WIDE, int CTAS>
 cudaError_t launch_inst(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmC0,
@@ -664,7 +687,7 @@ cudaError_t launch_inst(const CUtensorMap& tmA, const CUtensorMap& tmB, const CU
   // persistent: one CTA (or one pair) per SM (pair of SMs), each walking its work list
   const int tiles_m = (M + BM * CTAS - 1) / (BM * CTAS), tiles_n = (N + BN - 1) / BN;
   const int tiles_m2 = sec.M > 0 ? (sec.M + BM * CTAS - 1) / (BM * CTAS) : 0, tiles_n2 = sec.M > 0 ? (sec.N + BN - 1) / BN : 0;
-  const int units = tiles_m * tiles_n + tiles_m2 * tiles_n2;
+  const int units = tiles_m * tiles_n + tiles_m2 * tiles_n2 * (sec.out3 != nullptr ? 2 : 1);
   const int slots = device_sm_count() / CTAS;
   const int P = sk_tail > 0 ? slots : (units < slots ? units : slots);
   const int dp_tiles = sk_tail > 0 ? units - sk_tail : units;
@@ -682,9 +705,11 @@ cudaError_t launch_inst(const CUtensorMap& tmA, const CUtensorMap& tmB, const CU
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  const bool second_maps = sec.M > 0 || sec.maps;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmC0, tmC1, sec.M > 0 ? sec.A : tmA, second_maps ? sec.B : tmB,
-                                     second_maps ? sec.C : tmC0, M, N, K, sec.M, sec.N, 8, dp_tiles, sk_split, ep);
+  const bool second_maps = sec.M > 0 || sec.maps, concat = sec.k_switch != 0x7fffffff, third = sec.out3 != nullptr;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmC0, tmC1, sec.M > 0 || concat ? sec.A : tmA,
+                                     second_maps || concat ? sec.B : tmB, second_maps ? sec.C : tmC0, third ? sec.A3 : tmA,
+                                     third ? sec.C3 : tmC0, M, N, K, sec.M, sec.N, third ? 1 : 0, sec.k_switch, 8, dp_tiles,
+                                     sk_split, ep);
   count_launches(1);
   if (e == cudaSuccess && sk_tail > 0) {
     cudaLaunchConfig_t fcfg = {};
@@ -695,13 +720,22 @@ cudaError_t launch_inst(const CUtensorMap& tmA, const CUtensorMap& tmB, const CU
     fcfg.numAttrs = 1;
     e = cudaLaunchKernelEx(&fcfg, tail_fixup_kernel<BN, CTAS>, M, N, dp_tiles, sk_tail, sk_split, tiles_m, tiles_n, 8,
                            static_cast<const float*>(ep.sk_scratch), ep.out, static_cast<int>(ep.out_fp32),
-                           static_cast<int>(ep.accumulate), sec.M, sec.N, tiles_m2, tiles_n2, sec.out);
+                           static_cast<int>(ep.accumulate), sec.M, sec.N, tiles_m2, tiles_n2, sec.out, sec.out3);
     count_launches(1);
   }
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-struct SecondProduct { int M = 0, N = 0; const void* A = nullptr; const void* B = nullptr; void* out = nullptr; };
+// M > 0: a second product (out3: and a third, A3 with the same B); concat: C = A B^T + second A B^T.
+struct SecondProduct {
+  int M = 0, N = 0;
+  const void* A = nullptr;
+  const void* B = nullptr;
+  void* out = nullptr;
+  const void* A3 = nullptr;
+  void* out3 = nullptr;
+  bool concat = false;
+};
 
 template <bool A_MN, bool B_MN, int KIND, int CTAS, int BN = 256>
 cudaError_t launch_bn(const void* A, const void* B, int M, int N, int K, const EpiParams& ep,
@@ -725,13 +759,25 @@ cudaError_t launch_bn(const void* A, const void* B, int M, int N, int K, const E
       okC = okC && (A_MN ? encode_map(&sec.A, second.A, K, second.M, BK) : encode_map(&sec.A, second.A, second.M, K, BM));
       okC = okC && (B_MN ? encode_map(&sec.B, second.B, K, second.N, BK) : encode_map(&sec.B, second.B, second.N, K, BN / CTAS));
       okC = okC && encode_out_map(&sec.C, second.out, second.M, second.N, ep.out_fp32 != 0);
+      if (second.out3 != nullptr) {
+        sec.out3 = second.out3;
+        okC = okC && (A_MN ? encode_map(&sec.A3, second.A3, K, second.M, BK) : encode_map(&sec.A3, second.A3, second.M, K, BM));
+        okC = okC && encode_out_map(&sec.C3, second.out3, second.M, second.N, ep.out_fp32 != 0);
+      }
+    }
+    if (second.concat) {
+      // each contraction ends with its own (zero-filled) ragged block
+      sec.k_switch = (K + BK - 1) / BK;
+      okC = okC && (A_MN ? encode_map(&sec.A, second.A, K, M, BK) : encode_map(&sec.A, second.A, M, K, BM));
+      okC = okC && (B_MN ? encode_map(&sec.B, second.B, K, N, BK) : encode_map(&sec.B, second.B, N, K, BN / CTAS));
+      K = 2 * sec.k_switch * BK;
     }
     // The last round costs ceil(tail * split / slots) / split tile times instead of one.
     // Worth it when that saves clearly more than the partial tiles and the fix-up launch
     // cost (10-25 us together); a tile time is ~ 2 TM BN K flops at ~11 TFLOP/s per SM.
     constexpr int TM = BM * CTAS;
     const int units = ((M + TM - 1) / TM) * ((N + BN - 1) / BN) +
-                      (second.M > 0 ? ((second.M + TM - 1) / TM) * ((second.N + BN - 1) / BN) : 0);
+                      (second.M > 0 ? ((second.M + TM - 1) / TM) * ((second.N + BN - 1) / BN) : 0) * (second.out3 != nullptr ? 2 : 1);
     const int slots = device_sm_count() / CTAS;
     const int k_blocks = (K + BK - 1) / BK;
     const int tail = units % slots;
@@ -801,16 +847,26 @@ cudaError_t launch_tc_gemm_dagger(int M, int N, int K, const void* A, const void
 }
 
 cudaError_t launch_tc_gemm_token_pair(int K, int M1, int N1, const void* A1, const void* B1, void* out1, int M2,
-                                      int N2, const void* A2, const void* B2, void* out2, const EpiParams& ep,
-                                      bool pair, cudaStream_t stream) {
+                                      int N2, const void* A2, const void* B2, void* out2, const void* A3, void* out3,
+                                      const EpiParams& ep, bool pair, cudaStream_t stream) {
   if (K <= 0 || M1 <= 0 || N1 <= 0 || M2 <= 0 || N2 <= 0) return cudaErrorNotSupported;
   if ((M1 % 8) || (N1 % 8) || (M2 % 8) || (N2 % 8)) return cudaErrorNotSupported;
   EpiParams p = ep;
   p.out = out1;
   SecondProduct second;
-  second.M = M2; second.N = N2; second.A = A2; second.B = B2; second.out = out2;
+  second.M = M2; second.N = N2; second.A = A2; second.B = B2; second.out = out2; second.A3 = A3; second.out3 = out3;
   if (pair) return launch_bn<true, true, kEpiStore, 2>(A1, B1, M1, N1, K, p, second, stream);
   return launch_bn<true, true, kEpiStore, 1>(A1, B1, M1, N1, K, p, second, stream);
+}
+
+cudaError_t launch_tc_gemm_sum(int M, int N, int K, const void* A1, const void* B1, const void* A2, const void* B2,
+                               const EpiParams& ep, bool pair, cudaStream_t stream) {
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  if (K <= 0 || (N % 8) || (K % 8)) return cudaErrorNotSupported;
+  SecondProduct second;
+  second.A = A2; second.B = B2; second.concat = true;
+  if (pair) return launch_bn<false, true, kEpiStore, 2>(A1, B1, M, N, K, ep, second, stream);
+  return launch_bn<false, true, kEpiStore, 1>(A1, B1, M, N, K, ep, second, stream);
 }
 
 void* tensor_map_encode_fn() {

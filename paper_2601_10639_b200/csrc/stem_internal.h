@@ -105,14 +105,20 @@ cudaError_t launch_split_gemm(const SplitProduct& p, const SplitProduct& second,
 cudaError_t launch_tc_gemm(int M, int N, int K, const void* A, bool a_mn, const void* B,
                            bool b_mn, EpiKind kind, const EpiParams& ep, bool pair, cudaStream_t stream);
 
-// Two token-contracted products in one launch (the two weight gradients of the layer):
-//   out1[m,n] = sum_k A1(k,m) B1(k,n)   and   out2[m,n] = sum_k A2(k,m) B2(k,n),
-// all four operands stored [K, .] row-major (MN-major), both outputs of ep.out_fp32's type, the
-// same ep.accumulate.  Their tiles share one work list, so the pair fills the SMs where each
-// product alone leaves some idle; ep.out is ignored (out1 / out2 are the outputs).
+// Two or three token-contracted products in one launch (the layer's weight gradients):
+//   out1[m,n] = sum_k A1(k,m) B1(k,n),   out2[m,n] = sum_k A2(k,m) B2(k,n)   and, with out3 not NULL,
+//   out3[m,n] = sum_k A3(k,m) B2(k,n),
+// all operands stored [K, .] row-major (MN-major), all outputs of ep.out_fp32's type, the same
+// ep.accumulate.  Their tiles share one work list, so together they fill the SMs where each product
+// alone leaves some idle; ep.out is ignored.
 cudaError_t launch_tc_gemm_token_pair(int K, int M1, int N1, const void* A1, const void* B1, void* out1, int M2,
-                                      int N2, const void* A2, const void* B2, void* out2, const EpiParams& ep,
-                                      bool pair, cudaStream_t stream);
+                                      int N2, const void* A2, const void* B2, void* out2, const void* A3, void* out3,
+                                      const EpiParams& ep, bool pair, cudaStream_t stream);
+
+// C[m,n] = sum_k A1[m,k] B1[k,n] + sum_k A2[m,k] B2[k,n]: one contraction over both pairs of operands
+// (A K-major, B MN-major), plain store.
+cudaError_t launch_tc_gemm_sum(int M, int N, int K, const void* A1, const void* B1, const void* A2, const void* B2,
+                               const EpiParams& ep, bool pair, cudaStream_t stream);
 
 // The dagger variant's gate and up products of the same x tile in one launch (CTA pairs, two
 // accumulators): G = A B_gate^T, Up = A B_up^T, then U = Up + E[ids], H = SiLU(G) * U in the
