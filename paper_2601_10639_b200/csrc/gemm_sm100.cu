@@ -737,6 +737,26 @@ struct SecondProduct {
   bool concat = false;
 };
 
+// Tiles of the ragged last round, and pieces per tile along k (1: the round stays whole).  The last
+// round costs ceil(tail * pieces / slots) / pieces tile times instead of one.  Worth it when that saves
+// clearly more than the partial tiles and the fix-up launch cost (10-25 us together); a tile time is
+// ~ 2 TM BN K flops at ~11 TFLOP/s per SM.
+struct TailSplit { int tail, pieces; };
+TailSplit split_tail(int units, int K, int bn, int ctas, const EpiParams& ep) {
+  const int tm = BM * ctas, slots = device_sm_count() / ctas, k_blocks = (K + BK - 1) / BK, tail = units % slots;
+  const size_t slot_bytes = static_cast<size_t>(tm) * bn * sizeof(float);
+  const double tile_us = 2.0 * tm * bn * static_cast<double>(K) / (11.0e6 * ctas);
+  if (tail == 0 || ep.sk_scratch == nullptr) return {tail, 1};
+  int best = 1;
+  double best_cost = 1.0;
+  for (int sp = 2; sp <= kMaxSplit; ++sp) {
+    if (static_cast<size_t>(tail) * sp * slot_bytes > ep.sk_bytes || k_blocks / sp < 4) break;
+    const double cost = static_cast<double>((tail * sp + slots - 1) / slots) / sp;
+    if (cost < best_cost - 0.04) { best_cost = cost; best = sp; }
+  }
+  return {tail, (1.0 - best_cost) * tile_us > 25.0 ? best : 1};
+}
+
 template <bool A_MN, bool B_MN, int KIND, int CTAS, int BN = 256>
 cudaError_t launch_bn(const void* A, const void* B, int M, int N, int K, const EpiParams& ep,
                       const SecondProduct& second, cudaStream_t stream) {
@@ -772,30 +792,14 @@ cudaError_t launch_bn(const void* A, const void* B, int M, int N, int K, const E
       okC = okC && (B_MN ? encode_map(&sec.B, second.B, K, N, BK) : encode_map(&sec.B, second.B, N, K, BN / CTAS));
       K = 2 * sec.k_switch * BK;
     }
-    // The last round costs ceil(tail * split / slots) / split tile times instead of one.
-    // Worth it when that saves clearly more than the partial tiles and the fix-up launch
-    // cost (10-25 us together); a tile time is ~ 2 TM BN K flops at ~11 TFLOP/s per SM.
     constexpr int TM = BM * CTAS;
     const int units = ((M + TM - 1) / TM) * ((N + BN - 1) / BN) +
                       (second.M > 0 ? ((second.M + TM - 1) / TM) * ((second.N + BN - 1) / BN) : 0) * (second.out3 != nullptr ? 2 : 1);
-    const int slots = device_sm_count() / CTAS;
-    const int k_blocks = (K + BK - 1) / BK;
-    const int tail = units % slots;
-    const size_t slot_bytes = static_cast<size_t>(TM) * BN * sizeof(float);
-    const double tile_us = 2.0 * TM * BN * static_cast<double>(K) / (11.0e6 * CTAS);
-    if (tail > 0 && ep.sk_scratch != nullptr) {
-      int best = 1;
-      double best_cost = 1.0;
-      for (int sp = 2; sp <= kMaxSplit; ++sp) {
-        if (static_cast<size_t>(tail) * sp * slot_bytes > ep.sk_bytes || k_blocks / sp < 4) break;
-        const double cost = static_cast<double>((tail * sp + slots - 1) / slots) / sp;
-        if (cost < best_cost - 0.04) { best_cost = cost; best = sp; }
-      }
-      if (best > 1 && (1.0 - best_cost) * tile_us > 25.0) {
-        sk_tail = tail;
-        sk_split = best;
-        okC = okC && encode_out_map(&tmC1, ep.sk_scratch, tail * best * TM, BN, true);
-      }
+    const TailSplit ts = split_tail(units, K, BN, CTAS, ep);
+    if (ts.pieces > 1) {
+      sk_tail = ts.tail;
+      sk_split = ts.pieces;
+      okC = okC && encode_out_map(&tmC1, ep.sk_scratch, sk_tail * sk_split * TM, BN, true);
     }
   } else {
     okC = encode_out_map(&tmC0, ep.H, M, N, false);
@@ -811,12 +815,14 @@ cudaError_t launch_bn(const void* A, const void* B, int M, int N, int K, const E
 template <bool A_MN, bool B_MN, int KIND>
 cudaError_t launch_ctas(const void* A, const void* B, int M, int N, int K, const EpiParams& ep, bool pair,
                         cudaStream_t stream) {
-  if constexpr (KIND == kEpiGate) {
-    // A decode-sized batch (one row of tiles) leaves most CTA pairs without a tile and makes the
-    // one tile a pair has a serial chain of load, multiply, epilogue.  Halving the tile width
-    // doubles the pairs at work and halves that chain; beyond 256 rows the extra passes over x
-    // cost more than they save (measured: 256 rows 22.6 -> 20.5 us, 512 rows 23.8 -> 28.8 us).
-    if (pair && M <= 256 && (N + 127) / 128 <= device_sm_count() / 2)
+  if constexpr (!A_MN) {
+    // A batch whose tiles leave half of the CTA pairs without one: tiles of half the width put twice as
+    // many pairs to work and halve each one's chain of load, multiply, epilogue, at 4/3 of the cost per
+    // flop.  (Where the contraction is long enough to be cut along k instead, that gains more.)
+    // Forward at 1024 x 2816: 300 rows 30.6 -> 25.6 us, 1531 rows 33.3 -> 30.8, 2400 rows alike.
+    const int slots = device_sm_count() / 2, units = ((M + 2 * BM - 1) / (2 * BM)) * ((N + 127) / 128);
+    if (pair && units <= slots &&
+        (KIND != kEpiStore || split_tail(((M + 2 * BM - 1) / (2 * BM)) * ((N + 255) / 256), K, 256, 2, ep).pieces == 1))
       return launch_bn<A_MN, B_MN, KIND, 2, 128>(A, B, M, N, K, ep, SecondProduct{}, stream);
   }
   if (pair) return launch_bn<A_MN, B_MN, KIND, 2>(A, B, M, N, K, ep, SecondProduct{}, stream);

@@ -1,6 +1,6 @@
 """bf16 layers on few rows (decode steps, short prompts) vs the CPU checker: the weight-streaming kernels at
 the edges of their padding (16 and 32 rows), of the batch they take, of W's 128-row tiles and 64-wide k blocks
-(one block, fewer blocks than a cluster has CTAs, a ragged last one)."""
+(one block, fewer blocks than a cluster has CTAs, a ragged last one), and the half-width tiles of the general kernel."""
 import numpy as np
 import pytest
 import torch
@@ -9,7 +9,7 @@ from oracle import stem_oracle as O
 from paper_2601_10639_b200 import binding as B
 from paper_2601_10639_b200 import runner, synth
 from parity_measures import TOL_BF16, assert_close
-from test_gpu_parity import _np
+from test_gpu_parity import _full_parity, _np
 
 pytestmark = pytest.mark.gpu
 
@@ -31,6 +31,12 @@ def test_forward_few_rows(T, d, F):
     st.bufs["y"].fill_(float("nan"))
     st.forward(save=False)                       # H in the workspace, G nowhere
     assert st.status() == B.OK and torch.equal(st.bufs["y"], y)
+
+
+@pytest.mark.parametrize("T,d,F", [(300, 264, 520), (700, 1024, 2816)])
+def test_layer_half_width_tiles(T, d, F):
+    w = synth.Workload("t", T, d, F, 300, "bf16", "zipf")
+    _full_parity(w, synth.make_inputs(w, seed=43), B.DTYPE_BF16, TOL_BF16)
 
 
 def test_few_rows_bad_id_is_clamped_and_reported():
