@@ -21,8 +21,8 @@
 // produced the operand (EpiParams::H3, G3).  Splitting inside the contraction instead, on the way from
 // global to shared memory, converts every operand once per tile row or column that uses it and is bound
 // by that.  Measured, a layer's training step at 2048 positions, d_model 1024, d_ff 2816: 3600 us on the
-// FMA kernel, 787 us splitting inside, 531 us so (down, dx 63 us = 187 TFLOP/s each; gate 111, dH 128,
-// the weight gradients 126); at 256 positions, 256, 688: 237, 72 and 80 us.  Error against 64 bits:
+// FMA kernel, 787 us splitting inside, 511 us so (down, dx 62 us = 192 TFLOP/s each; gate 109, dH 117,
+// the weight gradients 125); at 256 positions, 256, 688: 237, 72 and 74 us.  Error against 64 bits:
 // 0.2 - 0.5 of the FMA kernel's for K >= 128, alike at K = 8.
 //
 // A tile is 128 * CTAS rows x BN columns.  CTAS = 2: a pair of CTAs shares each MMA (cta_group::2), each
@@ -152,15 +152,14 @@ __device__ __forceinline__ bool needs_chain(float v) {
   constexpr uint32_t kTiny = 29u << 23;   // 2^-98
   return u - kTiny > 0x7F7FFFFFu - kTiny && u != 0;
 }
-// The plain chain of FMAs for them; a[i] is column n + i of row m.  (One loop over the marked columns:
-// a copy of the chain per column would be most of the kernel's code.  A NaN stays one, so the chain
-// ends there.)
+// The plain chain of FMAs for them; a[i] is column n + i of row m.  (A NaN stays one, so the chain ends
+// there.)
 template <bool A_MN, bool B_MN>
-__device__ __forceinline__ void redo_in_fp32(const Product& pr, int K, int m, int n, float (&a)[32]) {
+__device__ __forceinline__ void redo_in_fp32(const Product& pr, int K, int m, int n, int have, float (&a)[8]) {
   uint32_t marked = 0;
 #pragma unroll
-  for (int i = 0; i < 32; ++i)
-    if (needs_chain(a[i]) && n + i < pr.N) marked |= 1u << i;
+  for (int i = 0; i < 8; ++i)
+    if (needs_chain(a[i]) && i < have) marked |= 1u << i;
   while (marked != 0) {
     const int i = __ffs(marked) - 1;
     marked &= marked - 1;
@@ -170,7 +169,7 @@ __device__ __forceinline__ void redo_in_fp32(const Product& pr, int K, int m, in
       acc = fmaf(A_MN ? pr.A[static_cast<size_t>(k) * pr.M + m] : pr.A[static_cast<size_t>(m) * K + k],
                  B_MN ? pr.B[static_cast<size_t>(k) * pr.N + n + i] : pr.B[static_cast<size_t>(n + i) * K + k], acc);
 #pragma unroll
-    for (int j = 0; j < 32; ++j)
+    for (int j = 0; j < 8; ++j)
       if (j == i) a[j] = acc;
   }
 }
@@ -216,58 +215,43 @@ __device__ __forceinline__ void store_parts8(const Parts& parts, int m, int n, i
   }
 }
 
-// The operands that the fused step needs for 32 consecutive columns (n_cols of which are this thread's)
-// of one row: the table row (or addend) and the saved G.
+// The operands that the fused step needs for eight consecutive columns (have of them exist) of one row: the
+// table row (or addend) and the saved G.
 template <int KIND>
-__device__ __forceinline__ void load_operands(const EpiParams& ep, const Product& pr, int m, int n, int n_cols, int row_id,
-                                              float (&e)[32], float (&g)[32]) {
-  if (KIND == kEpiStore) return;
-  const float* e_row = static_cast<const float*>(ep.E) + static_cast<size_t>(row_id) * pr.N + n;
-  const float* g_row = static_cast<const float*>(ep.Gin) + static_cast<size_t>(m) * pr.N + n;
-#pragma unroll
-  for (int c = 0; c < 32; c += 8) {
-    const int have = min(n_cols, pr.N - n) - c;
-    if (have > 0) {
-      load8(e_row + c, pr.wide, have, e + c);
-      if (KIND == kEpiDH) load8(g_row + c, pr.wide, have, g + c);
-    }
-  }
+__device__ __forceinline__ void load_operands(const EpiParams& ep, const Product& pr, int m, int n, int have, int row_id,
+                                              float (&e)[8], float (&g)[8]) {
+  if (KIND == kEpiStore || have <= 0) return;
+  load8(static_cast<const float*>(ep.E) + static_cast<size_t>(row_id) * pr.N + n, pr.wide, have, e);
+  if (KIND == kEpiDH) load8(static_cast<const float*>(ep.Gin) + static_cast<size_t>(m) * pr.N + n, pr.wide, have, g);
 }
 
 // Fused elementwise step on them (formulas: EpiParams).
 template <int KIND>
-__device__ __forceinline__ void epilogue32(const EpiParams& ep, const Product& pr, int m, int n, int n_cols,
-                                           const float (&a)[32], const float (&e)[32], const float (&g)[32]) {
+__device__ __forceinline__ void epilogue8(const EpiParams& ep, const Product& pr, int m, int n, int have, const float (&a)[8],
+                                          const float (&e)[8], const float (&g)[8]) {
+  const size_t o = static_cast<size_t>(m) * pr.N + n;
+  float r[8], r2[8];
+  if (KIND == kEpiStore && ep.accumulate) load8(pr.out + o, pr.wide, have, r2);
 #pragma unroll
-  for (int c = 0; c < 32; c += 8) {
-    const int have = min(n_cols, pr.N - n) - c;
-    if (have <= 0) break;
-    const size_t o = static_cast<size_t>(m) * pr.N + n + c;
-    float r[8], r2[8];
-    if (KIND == kEpiStore && ep.accumulate) {
-      load8(pr.out + o, pr.wide, have, r2);
+  for (int i = 0; i < 8; ++i) {
+    const float x = a[i];
+    if (KIND == kEpiStore) {
+      r[i] = ep.accumulate ? x + r2[i] : x;
+    } else if (KIND == kEpiAdd) {
+      r[i] = x + e[i];
+    } else if (KIND == kEpiGate) {
+      r[i] = x * sigmoid_f32(x) * e[i];
+      r2[i] = x;
+    } else {
+      const float s = sigmoid_f32(g[i]);
+      r[i] = x * (g[i] * s);                                       // dU
+      r2[i] = x * e[i] * (s * (1.0f + g[i] * (1.0f - s)));         // dG
     }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float x = a[c + i];
-      if (KIND == kEpiStore) {
-        r[i] = ep.accumulate ? x + r2[i] : x;
-      } else if (KIND == kEpiAdd) {
-        r[i] = x + e[c + i];
-      } else if (KIND == kEpiGate) {
-        r[i] = x * sigmoid_f32(x) * e[c + i];
-        r2[i] = x;
-      } else {
-        const float gi = g[c + i], s = sigmoid_f32(gi);
-        r[i] = x * (gi * s);                                       // dU
-        r2[i] = x * e[c + i] * (s * (1.0f + gi * (1.0f - s)));     // dG
-      }
-    }
-    store8((KIND == kEpiStore ? pr.out : static_cast<float*>(ep.H)) + o, pr.wide, have, r);
-    if (KIND == kEpiGate && ep.H3.base != nullptr) store_parts8(ep.H3, m, n + c, have, r);
-    if (KIND == kEpiDH || (KIND == kEpiGate && ep.G != nullptr)) store8(static_cast<float*>(ep.G) + o, pr.wide, have, r2);
-    if (KIND == kEpiDH && ep.G3.base != nullptr) store_parts8(ep.G3, m, n + c, have, r2);
   }
+  store8((KIND == kEpiStore ? pr.out : static_cast<float*>(ep.H)) + o, pr.wide, have, r);
+  if (KIND == kEpiGate && ep.H3.base != nullptr) store_parts8(ep.H3, m, n, have, r);
+  if (KIND == kEpiDH || (KIND == kEpiGate && ep.G != nullptr)) store8(static_cast<float*>(ep.G) + o, pr.wide, have, r2);
+  if (KIND == kEpiDH && ep.G3.base != nullptr) store_parts8(ep.G3, m, n, have, r2);
 }
 
 template <int KIND>
@@ -439,7 +423,7 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
     const int half = (warp - 2) >> 2;       // which half of the tile's columns it handles
     const int r = q * 32 + lane;            // row among this CTA's 128
     int buf = 0; uint32_t bph = 0;
-    float acc[kCols / 32][32], e[32], g[32];
+    float acc[kCols], e[8], g[8];
     const int share = kCols / ksplit;       // columns of a tile that this thread finishes
     int id = 0;
     for (int tile = tile0; ok && tile < num_tiles; tile += tile_step) {
@@ -448,11 +432,11 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
       const int tt = second ? tile - tiles1 : tile, tm = second ? tiles_m2 : tiles_m1;
       const int m = tt % tm * TM + rank * BM + r, n0 = tt / tm * BN + half * kCols;
 #pragma unroll
-      for (int c = 0; c < kCols; ++c) acc[c / 32][c % 32] = 0.0f;
+      for (int c = 0; c < kCols; ++c) acc[c] = 0.0f;
       // the epilogue's first operands are on their way while the blocks are summed
       if (KIND != kEpiStore && m < pr.M) {
         id = table_row<KIND>(ep, m);
-        load_operands<KIND>(ep, pr, m, n0 + slice * share, share, id, e, g);
+        load_operands<KIND>(ep, pr, m, n0 + slice * share, min(share, pr.N - n0 - slice * share), id, e, g);
       }
       for (int kb = kb0; kb < kb1; ++kb) {
         bool mine = ptx::mbar_wait_bounded(tfull_bar(buf), bph, abort_flag, kWaitLimitCycles);
@@ -476,18 +460,25 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
             }
           }
 #pragma unroll
-          for (int i = 0; i < 32; ++i) acc[c / 32][i] += __uint_as_float(v[i]);
+          for (int i = 0; i < 32; ++i) acc[c + i] += __uint_as_float(v[i]);
         }
         if (++buf == BUFS) { buf = 0; bph ^= 1u; }
       }
       if (!ok) break;
       if (ksplit == 1) {
+        // Eight columns at a time in a rolled loop, the sums moving down: unrolled over the columns this is
+        // some 3000 instructions that a launch has to fetch first (layer of 256 rows: 79.5 -> 75 us rolled).
         if (m < pr.M) {
+#pragma unroll 1
+          for (int n = n0; n < min(n0 + kCols, pr.N); n += 8) {
+            float a8[8], e8[8], g8[8];
 #pragma unroll
-          for (int c = 0; c < kCols; c += 32) {
-            if (c > 0) load_operands<KIND>(ep, pr, m, n0 + c, 32, id, e, g);
-            redo_in_fp32<A_MN, B_MN>(pr, K, m, n0 + c, acc[c / 32]);
-            epilogue32<KIND>(ep, pr, m, n0 + c, 32, acc[c / 32], e, g);
+            for (int i = 0; i < 8; ++i) { a8[i] = acc[i]; e8[i] = e[i]; g8[i] = g[i]; }
+            load_operands<KIND>(ep, pr, m, n + 8, min(n0 + kCols, pr.N) - n - 8, id, e, g);
+            redo_in_fp32<A_MN, B_MN>(pr, K, m, n, pr.N - n, a8);
+            epilogue8<KIND>(ep, pr, m, n, pr.N - n, a8, e8, g8);
+#pragma unroll
+            for (int i = 0; i + 8 < kCols; ++i) acc[i] = acc[i + 8];
           }
         }
       } else {
@@ -495,7 +486,7 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
         // ring is free: leave the sums there, column by column (128 rows of a column side by side).
         float* part = reinterpret_cast<float*>(base_ptr) + static_cast<size_t>(half) * kCols * BM + r;
 #pragma unroll
-        for (int c = 0; c < kCols; ++c) part[c * BM] = acc[c / 32][c % 32];
+        for (int c = 0; c < kCols; ++c) part[c * BM] = acc[c];
       }
     }
     if (ksplit > 1) {
@@ -508,17 +499,25 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
       const int m = tt % tm * TM + rank * BM + r, n0 = tt / tm * BN + half * kCols + slice * share;
       if (ok && m < pr.M) {
         const uint32_t mine = base + 4u * (static_cast<uint32_t>(half * kCols + slice * share) * BM + r);
-        float v[32];
+        const int end = min(n0 + share, pr.N);
+#pragma unroll 1
+        for (int n = n0; n < end; n += 8) {
+          float a8[8], e8[8], g8[8];
 #pragma unroll
-        for (int c = 0; c < 32; ++c) v[c] = 0.0f;
-        for (int k = 0; k < ksplit; ++k) {
-          const uint32_t src = ptx::mapa(mine, k * CTAS + rank);
+          for (int i = 0; i < 8; ++i) { a8[i] = 0.0f; e8[i] = e[i]; g8[i] = g[i]; }
+          load_operands<KIND>(ep, pr, m, n + 8, end - n - 8, id, e, g);
+#pragma unroll 2
+          for (int k = 0; k < ksplit; ++k) {
+            const uint32_t src = ptx::mapa(mine + 4u * BM * (n - n0), k * CTAS + rank);
+            float v[8];
 #pragma unroll
-          for (int c = 0; c < 32; ++c)
-            if (c < share) v[c] += ptx::ld_shared_cluster_f32(src + 4u * BM * c);
+            for (int i = 0; i < 8; ++i) v[i] = n + i < end ? ptx::ld_shared_cluster_f32(src + 4u * BM * i) : 0.0f;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) a8[i] += v[i];
+          }
+          redo_in_fp32<A_MN, B_MN>(pr, K, m, n, end - n, a8);
+          epilogue8<KIND>(ep, pr, m, n, end - n, a8, e8, g8);
         }
-        redo_in_fp32<A_MN, B_MN>(pr, K, m, n0, v);
-        epilogue32<KIND>(ep, pr, m, n0, share, v, e, g);
       }
       __syncwarp();
     }
