@@ -1,10 +1,12 @@
 // Token-id deduplication: a stable LSD radix sort of (id, position) pairs, 8 bits per
 // pass (a count kernel and a scatter kernel per pass), followed by two kernels that mark
 // the head of every run of equal ids and emit the distinct ids, the run offsets and each
-// position's slot.  Batches of up to 1024 positions take a one-launch path (rank sort in
-// shared memory).  Integer-only: every output has exactly one correct value.
+// position's slot.  Batches of up to 256 positions take one launch of one CTA (rank sort in
+// shared memory), up to 16384 one launch of one cluster of CTAs (the radix sort with the pairs in
+// distributed shared memory).  Integer-only: every output has exactly one correct value.
 #include <mutex>
 
+#include "ptx_sm100.cuh"
 #include "stem_internal.h"
 
 namespace stem {
@@ -14,6 +16,10 @@ constexpr int kRadix = 256;
 constexpr int kWarps = 32;              // warps per CTA
 constexpr int kCtaThreads = kWarps * 32;
 constexpr int kMaxCtas = 64;
+// Which path a batch takes: up to here the rank sort of one CTA, up to kClusterMaxT one cluster, then the six
+// launches.  Measured, rank sort / cluster: 256 positions 11.0 us (the call itself) / the same, 512: 10.5 / 8.7,
+// 1000: 33.0 / 8.8; six launches / cluster: 1500: 13.2 / 8.1, 16384: 15.7 / 14.2, 32000: 17.0 / 20.8.
+constexpr int kRankSortMaxT = 256;
 
 // Work split: CTA c owns positions [c * 32 * epw, (c + 1) * 32 * epw), warp w of it the
 // w-th run of epw positions.  Few, large CTAs keep the cross-CTA bookkeeping (one digit
@@ -208,7 +214,7 @@ heads_write_kernel(int T, int per_cta, const int32_t* __restrict__ sorted_ids, c
   }
 }
 
-// A batch of at most kCtaThreads positions (decode steps) in one launch by one CTA: every
+// A batch of at most kRankSortMaxT positions (decode steps) in one launch by one CTA: every
 // thread ranks its own (id, position) pair against all others in shared memory, which is the
 // stable sort; run heads and slots follow from one block-wide scan.  Same outputs as the
 // radix path, without its six launch latencies.
@@ -275,6 +281,163 @@ dedup_small_kernel(int T, int V, const int32_t* __restrict__ ids, int32_t* __res
   }
 }
 
+// A batch of up to kClusterMaxT positions in one launch by one cluster of eight CTAs: CTA c keeps the c-th run
+// of `chunk` sorted (key, position) pairs in its shared memory; a radix pass counts digits, exchanges the
+// CTAs' counts and scatters the pairs through distributed shared memory; run heads and slots follow from
+// one scan over the cluster.  Same outputs as the radix path of six launches, for a cluster barrier
+// (well under a microsecond) in the place of each launch boundary and no round trip through memory.
+constexpr int kClusterCtas = 8;
+constexpr int kClusterMaxT = 16384;
+constexpr int kChunkMax = kClusterMaxT / kClusterCtas;
+struct ClusterSmem {
+  int2 pair[2][kChunkMax];       // key, position
+  int hist[kWarps][kRadix];
+  int digits[kRadix];            // this CTA's count of every digit
+  int warp_sum[kWarps];
+  int heads;
+};
+
+__device__ __forceinline__ uint32_t peer(const void* p, int cta) { return ptx::mapa(ptx::smem_u32(p), cta); }
+
+__global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kCtaThreads, 1)
+dedup_cluster_kernel(int T, int V, int chunk, int passes, const int32_t* __restrict__ ids, int32_t* __restrict__ unique_ids,
+                     int32_t* __restrict__ n_unique, int32_t* __restrict__ inverse, int32_t* __restrict__ perm,
+                     int32_t* __restrict__ seg_offsets, int32_t* status) {
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  ClusterSmem& sm = *reinterpret_cast<ClusterSmem*>(smem_raw);
+  const int cta = static_cast<int>(ptx::cluster_ctarank()), tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int first = cta * chunk, mine = max(0, min(chunk, T - first));       // positions of this CTA
+  const int epw = (chunk / 32 + kWarps - 1) / kWarps * 32;                   // ... of a warp (chunk: a multiple of 32)
+  const int begin = min(mine, w * epw), end = min(mine, begin + epw);
+  const unsigned lt_mask = (1u << lane) - 1u;
+  pdl_wait_then_release();
+  for (int i = begin + lane; i < end; i += 32) {
+    int key = ids[first + i];
+    if (key < 0 || key >= V) {
+      if (status != nullptr) { report_error(status, STEM_ERR_ID_RANGE, first + i); atomicAdd(status + 2, 1); }
+      key = clamp_id(key, V);
+    }
+    sm.pair[0][i] = make_int2(key, first + i);
+  }
+  int cur = 0;
+  for (int pass = 0; pass < passes; ++pass, cur ^= 1) {
+    const int shift = 8 * pass;
+    for (int i = lane; i < kRadix; i += 32) sm.hist[w][i] = 0;
+    __syncwarp();
+    for (int i = begin + lane; i < end; i += 32) atomicAdd(&sm.hist[w][(sm.pair[cur][i].x >> shift) & (kRadix - 1)], 1);
+    __syncthreads();
+    if (tid < kRadix) {
+      int sum = 0;
+#pragma unroll 8
+      for (int ww = 0; ww < kWarps; ++ww) sum += sm.hist[ww][tid];
+      sm.digits[tid] = sum;
+    }
+    __syncwarp();
+    ptx::cluster_sync();
+    // start of every (digit, warp): smaller digits first, then equal digits of earlier CTAs, then of earlier warps
+    int before = 0, total = 0, incl = 0;
+    if (tid < kRadix) {
+      int v[kClusterCtas];
+#pragma unroll
+      for (int c = 0; c < kClusterCtas; ++c) v[c] = ptx::ld_shared_cluster_s32(peer(&sm.digits[tid], c));
+#pragma unroll
+      for (int c = 0; c < kClusterCtas; ++c) { total += v[c]; before += c < cta ? v[c] : 0; }
+      incl = total;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+      }
+      if (lane == 31) sm.warp_sum[w] = incl;
+    }
+    __syncthreads();
+    if (tid < kRadix) {
+      int base = incl - total + before;
+      for (int ww = 0; ww < w; ++ww) base += sm.warp_sum[ww];
+      for (int ww = 0; ww < kWarps; ++ww) {
+        const int cnt = sm.hist[ww][tid];
+        sm.hist[ww][tid] = base;
+        base += cnt;
+      }
+    }
+    __syncthreads();
+    for (int i0 = begin; i0 < end; i0 += 32) {
+      const int i = i0 + lane;
+      const bool valid = i < end;
+      const int2 kv = valid ? sm.pair[cur][i] : make_int2(0, 0);
+      const int digit = (kv.x >> shift) & (kRadix - 1);
+      const unsigned peers = __match_any_sync(0xffffffffu, valid ? digit : (kRadix + lane));
+      const int rank = __popc(peers & lt_mask);
+      int dst = 0;
+      if (valid) dst = sm.hist[w][digit] + rank;
+      __syncwarp();
+      if (valid && rank == 0) sm.hist[w][digit] += __popc(peers);
+      __syncwarp();
+      if (valid) {
+        const int owner = dst / chunk;
+        ptx::st_shared_cluster_v2(peer(&sm.pair[cur ^ 1][dst - owner * chunk], owner), kv.x, kv.y);
+      }
+    }
+    __syncwarp();
+    ptx::cluster_sync();
+  }
+  // heads of runs of equal ids: a thread's positions, the CTA's, the cluster's
+  const int per_thread = (chunk + kCtaThreads - 1) / kCtaThreads;
+  const int p0 = min(mine, tid * per_thread), p1 = min(mine, p0 + per_thread);
+  int prev = -1;                                    // no id is negative here
+  if (p0 < p1 && first + p0 > 0)
+    prev = p0 > 0 ? sm.pair[cur][p0 - 1].x : ptx::ld_shared_cluster_s32(peer(&sm.pair[cur][chunk - 1].x, cta - 1));
+  int local = 0;
+  for (int p = p0, last = prev; p < p1; ++p) {
+    const int id = sm.pair[cur][p].x;
+    local += id != last ? 1 : 0;
+    last = id;
+  }
+  int incl = local;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
+  }
+  if (lane == 31) sm.warp_sum[w] = incl;
+  __syncthreads();
+  if (w == 0) {
+    int v = sm.warp_sum[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += u;
+    }
+    sm.warp_sum[lane] = v;
+    if (lane == 31) sm.heads = v;
+  }
+  __syncwarp();
+  ptx::cluster_sync();
+  int heads = incl - local + (w > 0 ? sm.warp_sum[w - 1] : 0), all = 0;
+  int counts[kClusterCtas];
+#pragma unroll
+  for (int c = 0; c < kClusterCtas; ++c) counts[c] = ptx::ld_shared_cluster_s32(peer(&sm.heads, c));
+#pragma unroll
+  for (int c = 0; c < kClusterCtas; ++c) { heads += c < cta ? counts[c] : 0; all += counts[c]; }
+  for (int p = p0; p < p1; ++p) {
+    const int2 kv = sm.pair[cur][p];
+    if (kv.x != prev) {
+      unique_ids[heads] = kv.x;
+      seg_offsets[heads] = first + p;
+      ++heads;
+      prev = kv.x;
+    }
+    perm[first + p] = kv.y;
+    if (inverse) inverse[kv.y] = heads - 1;
+  }
+  if (cta == 0 && tid == 0) {
+    *n_unique = all;
+    seg_offsets[all] = T;
+  }
+  __syncwarp();
+  ptx::cluster_sync();      // no CTA leaves while another reads its shared memory
+}
+
 __global__ void empty_dedup_kernel(int32_t* n_unique, int32_t* seg_offsets) {
   *n_unique = 0;
   seg_offsets[0] = 0;
@@ -334,7 +497,30 @@ cudaError_t launch_dedup(int T, int V, const int32_t* ids, int32_t* unique_ids, 
     count_launches(1);
     return cudaGetLastError();
   }
-  if (T <= kCtaThreads) {
+  if (T > kRankSortMaxT && T <= kClusterMaxT) {
+    static PerDeviceOnce configured;
+    if (cudaError_t ce = configured.run([] {
+          return cudaFuncSetAttribute(dedup_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      static_cast<int>(sizeof(ClusterSmem)));
+        }))
+      return ce;
+    const int chunk = ((T + kClusterCtas - 1) / kClusterCtas + 31) / 32 * 32;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kClusterCtas);
+    cfg.blockDim = dim3(kCtaThreads);
+    cfg.dynamicSmemBytes = sizeof(ClusterSmem);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, dedup_cluster_kernel, T, V, chunk, (key_bits(V) + 7) / 8, ids, unique_ids, n_unique,
+                                       inverse, perm, seg_offsets, status);
+    count_launches(1);
+    return e != cudaSuccess ? e : cudaGetLastError();
+  }
+  if (T <= kRankSortMaxT) {
     cudaError_t e = launch_chained(dedup_small_kernel, 1, kCtaThreads, stream, T, V, ids, unique_ids, n_unique, inverse,
                                    perm, seg_offsets, status);
     count_launches(1);

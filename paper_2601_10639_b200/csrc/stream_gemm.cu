@@ -418,12 +418,17 @@ cudaError_t launch_stream_gemm(int T, int F, int K, const void* X, const void* W
   return launch_inst<kEpiStore, 1>(X, W, T, F, K, pl, ep, stream);
 }
 
-// Above 128 rows a CTA has no room for a second one beside it, and the exchange (fp32 sums of the whole batch)
-// outweighs what is saved, but for a plain store of a short k range per CTA.  Measured, general kernel against
-// this one: gate, 144 rows: 20.4 / 22.6 us at 2048 x 8192, 14.4 / 16.4 at 1024 x 2816; down, 256 rows: 22.6 /
-// 18.4 us at 1024 x 2816 (6 blocks x 384 rows), 21.5 / 22.5 at 1536 x 5000 (10 x 384), 23.5 / 24.7 at 2048 x 8192.
+// Above 128 rows a CTA has no room for a second one beside it and the exchange (fp32 sums of the whole batch)
+// grows, so the lines depend on how much W there is to stream.  Measured, both forms of both kernels of a
+// forward pass, general / this one, 144, 192, 256 rows:
+//   2048 x 8192   31.7 / 25.7   33.0 / 27.4   34.0 / 32.9 us
+//   1800 x 6000   29.3 / 24.4   30.2 / 26.5   31.8 / 30.1
+//   1536 x 5000   24.5 / 22.5   27.3 / 25.0   28.4 / 28.7
+//   1024 x 2816   27.0 / 22.0   27.1 / 20.3   28.0 / 22.7, and 19.6, 20.5, 21.8 with only the second kernel so
+// (a plain store of a short k range per CTA: up to 3000 rows of operands, 6 blocks x 384 there).
 bool stream_gemm_pays(int T, int F, int K, EpiKind kind) {
-  if (T <= 128) return true;
+  const long long weights = static_cast<long long>(F) * K;
+  if (T <= 128 || (T <= 192 && weights >= 4000000) || (T <= kMaxT && weights >= 10000000)) return true;
   return kind == kEpiStore && T <= kMaxT && make_plan(T, F, K).rows <= 3000;
 }
 
