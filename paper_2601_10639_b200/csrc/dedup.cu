@@ -299,7 +299,8 @@ struct ClusterSmem {
 
 __device__ __forceinline__ uint32_t peer(const void* p, int cta) { return ptx::mapa(ptx::smem_u32(p), cta); }
 
-__global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kCtaThreads, 1)
+// 48 registers: with 64 a CTA takes a whole SM's and waits for one that no row mover has a CTA on.
+__global__ void __cluster_dims__(kClusterCtas, 1, 1) __maxnreg__(48)
 dedup_cluster_kernel(int T, int V, int chunk, int passes, const int32_t* __restrict__ ids, int32_t* __restrict__ unique_ids,
                      int32_t* __restrict__ n_unique, int32_t* __restrict__ inverse, int32_t* __restrict__ perm,
                      int32_t* __restrict__ seg_offsets, int32_t* status) {

@@ -4,7 +4,7 @@
 // 16-byte accesses, one row spread across the CTA; when the table is page-locked host
 // memory the loads cross the host link directly (no staging copy).  Kernels that talk to
 // host memory are meant to run beside the contraction kernels of another layer, which hold
-// every SM with one large CTA each: they are launched as kHostLinkCtas CTAs of
+// every SM with one large CTA each: they are launched as few CTAs of
 // kHostLinkThreads threads.  Even two of those fit next to a contraction CTA (registers,
 // threads; no shared memory), so the contraction never waits for an SM, and eight 16-byte
 // loads in flight per thread still cover several times the host link's bandwidth-delay
@@ -15,7 +15,11 @@ namespace stem {
 namespace {
 
 constexpr int kThreads = 256;          // device-to-device gathers
-constexpr int kHostLinkCtas = 32;
+constexpr int kHostLinkCtas = 32;      // write-back
+// Row gathers across the link take twice as many: while a write-back fills the link's other direction, the
+// requests of 32 CTAs (0.5 MB in flight) brought 13 MB in 1208 us, alone in 430.  A layer of 8192 positions, three
+// host tables, forward and backward: 2799 us with 32 CTAs, 2268 with 64, 2340 with 96, 2450 with 128.
+constexpr int kHostGatherCtas = 64;
 constexpr int kHostLinkThreads = 128;
 // A decode step's rows are few and the step waits for them: one CTA per row, so that no row's chain of
 // id, slot, host read waits for another's.  (With 32 CTAs such chains were five rows long at 147 rows.)
@@ -174,7 +178,7 @@ cudaError_t launch_gather_rows(int max_rows, int V, size_t row_bytes, const int3
   const int lanes_per_row = vec < threads ? vec : threads;
   const int rows_per_cta = threads / lanes_per_row;
   int blocks = (max_rows + rows_per_cta - 1) / rows_per_cta;
-  const int cap = max_rows <= kDecodeRows ? kDecodeRows : kHostLinkCtas;
+  const int cap = max_rows <= kDecodeRows ? kDecodeRows : kHostGatherCtas;
   if (blocks > cap) blocks = cap;
   if (!table_on_host) {
     // a device table: flat copy, as many CTAs as the largest possible count needs, up to 8 per SM
