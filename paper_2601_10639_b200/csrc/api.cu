@@ -298,7 +298,6 @@ int stem_ffn_forward(const stem_shape_t* shape, const void* x, const int32_t* id
       e = split3({x3, wg3, wd3}, st);
     }
     if (e != cudaSuccess) return cuda_fail(e);
-    gate.H3 = h3.p;
     {
       ProfScope prof("gate_gemm", st);
       e = split_gemm(T, F, d, x3, false, wg3, false, kEpiGate, gate, st);
@@ -306,6 +305,11 @@ int stem_ffn_forward(const stem_shape_t* shape, const void* x, const int32_t* id
     if (e != cudaSuccess) return cuda_fail(e);
     EpiParams down;
     down.out = y; down.status = status_of(ws);
+    {
+      ProfScope prof("split_operands", st);
+      e = split3({h3}, st);
+    }
+    if (e != cudaSuccess) return cuda_fail(e);
     ProfScope prof("down_gemm", st);
     e = split_gemm(T, d, F, h3, false, wd3, false, kEpiStore, down, st);
     return e == cudaSuccess ? STEM_OK : cuda_fail(e);
@@ -370,14 +374,18 @@ int stem_ffn_backward(const stem_shape_t* shape, const void* dy, const void* x, 
   if (split) {
     {
       ProfScope prof("split_operands", st);
-      // the operands of the outputs that are asked for; dG's parts come from the dH epilogue
+      // the operands of the outputs that are asked for
       Operand none{};
       e = split3({dy3, wd3, dW_gate ? x3 : none, dx ? wg3 : none, dW_down ? h3 : none}, st);
     }
     if (e != cudaSuccess) return cuda_fail(e);
-    if (dW_gate || dx) dh.G3 = dg3.p;
-    ProfScope prof("dh_gemm", st);
-    e = split_gemm(T, F, d, dy3, false, wd3, true, kEpiDH, dh, st);
+    {
+      ProfScope prof("dh_gemm", st);
+      e = split_gemm(T, F, d, dy3, false, wd3, true, kEpiDH, dh, st);
+    }
+    if (e != cudaSuccess) return cuda_fail(e);
+    ProfScope prof("split_operands", st);
+    if (dW_gate || dx) e = split3({dg3}, st);
   } else {
     ProfScope prof("dh_gemm", st);
     e = gemm(shape, T, F, d, dy, false, W_down, true, kEpiDH, dh, st);
@@ -537,7 +545,6 @@ int stem_dagger_forward(const stem_shape_t* shape, const void* x, const int32_t*
     {  // G = x W_gate^T, H = SiLU(G) (.) U: the gate epilogue with U as a [T, d_ff] "table" indexed by position
       EpiParams gate;
       gate.ids = nullptr; gate.E = U_save; gate.V = T; gate.H = H; gate.G = G_save; gate.status = status_of(ws);
-      if (split) gate.H3 = operand(ws, w.h3_off, H, T, F).p;
       ProfScope prof("gate_gemm", st);
       e = split ? split_gemm(T, F, d, x3, false, wg3, false, kEpiGate, gate, st)
                 : gemm(shape, T, F, d, x, false, W_gate, false, kEpiGate, gate, st);
@@ -549,7 +556,7 @@ int stem_dagger_forward(const stem_shape_t* shape, const void* x, const int32_t*
     EpiParams down;
     down.out = y; down.status = status_of(ws);
     ProfScope prof("down_gemm", st);
-    e = split3({wd3}, st);
+    e = split3({wd3, h3}, st);
     if (e == cudaSuccess) e = split_gemm(T, d, F, h3, false, wd3, false, kEpiStore, down, st);
     return e == cudaSuccess ? STEM_OK : cuda_fail(e);
   }
@@ -600,7 +607,6 @@ int stem_dagger_backward(const stem_shape_t* shape, const void* dy, const void* 
     ProfScope prof("dh_gemm", st);
     if (split) {
       Operand none{};
-      dh.G3 = dg3.p;
       e = split3({dy3, wd3, x3, wg3, dW_down ? h3 : none}, st);
       if (e == cudaSuccess) e = split_gemm(T, F, d, dy3, false, wd3, true, kEpiDH, dh, st);
     } else {
@@ -630,7 +636,7 @@ int stem_dagger_backward(const stem_shape_t* shape, const void* dy, const void* 
                          base + w.part_off, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }
-  if (split && (dW_up || dx) && (e = split3({du3, wu3}, st)) != cudaSuccess) return cuda_fail(e);
+  if (split && (dW_gate || dW_up || dx) && (e = split3({dg3, du3, wu3}, st)) != cudaSuccess) return cuda_fail(e);
   if (together) {
     EpiParams p; p.out_fp32 = grad_fp32; p.status = status_of(ws);
     p.accumulate = (shape->flags & STEM_FLAG_ACCUM_GRADS) != 0;

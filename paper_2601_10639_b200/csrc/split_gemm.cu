@@ -17,11 +17,12 @@
 // of both signs) or below 2^-98 (third parts below 2^-133 are lost, an error of up to K 2^-134 times
 // the other operand) is computed again from the fp32 operands as one chain of FMAs in ascending k.
 //
-// The parts come from split3_kernel, one launch for all operands of a call, or from the epilogue that
-// produced the operand (EpiParams::H3, G3).  Splitting inside the contraction instead, on the way from
+// The parts come from split3_kernel: one launch for the operands of a call, one for H or dG once they are
+// there.  (Written by the epilogue that makes H or dG instead, 16 bytes per row and instruction, they cost it
+// 24 us of 109 at 2048 x 2816 where the launch costs 10.)  Splitting inside the contraction instead, on the way from
 // global to shared memory, converts every operand once per tile row or column that uses it and is bound
 // by that.  Measured, a layer's training step at 2048 positions, d_model 1024, d_ff 2816: 3600 us on the
-// FMA kernel, 787 us splitting inside, 511 us so (down, dx 62 us = 192 TFLOP/s each; gate 109, dH 117,
+// FMA kernel, 787 us splitting inside, 494 us so (down, dx 62 us = 192 TFLOP/s each; gate 83, dH 94,
 // the weight gradients 125); at 256 positions, 256, 688: 237, 72 and 74 us.  Error against 64 bits:
 // 0.2 - 0.5 of the FMA kernel's for K >= 128, alike at K = 8.
 //
@@ -202,19 +203,6 @@ __device__ __forceinline__ void store8(float* p, bool wide, int have, const floa
   for (int h = 0; h < 8; h += 4)
     if (h < have) *reinterpret_cast<float4*>(p + h) = make_float4(x[h], x[h + 1], x[h + 2], x[h + 3]);
 }
-__device__ __forceinline__ void store_parts8(const Parts& parts, int m, int n, int have, const float (&r)[8]) {
-  uint32_t o[3][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) split_pair(r[2 * i], r[2 * i + 1], o[0][i], o[1][i], o[2][i]);
-  __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(parts.base) + static_cast<size_t>(m) * parts.pitch + n;
-  const size_t plane = static_cast<size_t>(parts.rows) * parts.pitch;
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    if (have >= 8) *reinterpret_cast<uint4*>(dst + s * plane) = make_uint4(o[s][0], o[s][1], o[s][2], o[s][3]);
-    else *reinterpret_cast<uint2*>(dst + s * plane) = make_uint2(o[s][0], o[s][1]);
-  }
-}
-
 // The operands that the fused step needs for eight consecutive columns (have of them exist) of one row: the
 // table row (or addend) and the saved G.
 template <int KIND>
@@ -249,9 +237,7 @@ __device__ __forceinline__ void epilogue8(const EpiParams& ep, const Product& pr
     }
   }
   store8((KIND == kEpiStore ? pr.out : static_cast<float*>(ep.H)) + o, pr.wide, have, r);
-  if (KIND == kEpiGate && ep.H3.base != nullptr) store_parts8(ep.H3, m, n, have, r);
   if (KIND == kEpiDH || (KIND == kEpiGate && ep.G != nullptr)) store8(static_cast<float*>(ep.G) + o, pr.wide, have, r2);
-  if (KIND == kEpiDH && ep.G3.base != nullptr) store_parts8(ep.G3, m, n, have, r2);
 }
 
 template <int KIND>

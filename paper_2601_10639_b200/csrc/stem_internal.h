@@ -38,13 +38,6 @@ __device__ __forceinline__ float sigmoid_f32(float g) { return 1.0f / (1.0f + ex
 // ---- epilogue descriptions (shared by the FMA and the tensor-core GEMM front ends) ---
 enum EpiKind : int { kEpiStore = 0, kEpiGate = 1, kEpiDH = 2, kEpiAdd = 3, kEpiDagger = 4 };
 
-// An fp32 matrix as the sum of three bf16 ones: [3][rows, cols], row pitch a multiple of 8 elements.
-struct Parts {
-  void* base = nullptr;
-  int rows = 0, cols = 0, pitch = 0;
-};
-inline size_t parts_bytes(size_t rows, size_t cols) { return align_up(3 * rows * ((cols + 7) / 8 * 8) * 2, 256); }
-
 struct EpiParams {
   // kEpiStore: out[m*ld + n] = acc              (out_fp32 selects fp32 or bf16/T storage)
   //            accumulate: out[m*ld + n] += acc   (gradient accumulation over micro-batches)
@@ -65,8 +58,6 @@ struct EpiParams {
   // kEpiDagger (two products of the same A tile, gate = acc and up = acc2):
   //            U = acc2 + E[ids[m], n]; H = SiLU(acc) * U; optional G = acc, optional U out
   void* U = nullptr;
-  // fp32 on the tensor cores, optional: the parts of H (kEpiGate) and of dG (kEpiDH) as well
-  Parts H3, G3;
   int32_t* status = nullptr;
   // kEpiStore, optional: scratch for partial tiles when the last round of tiles is split
   // along k (tc_gemm_scratch_bytes()); without it every tile is computed whole
@@ -81,8 +72,13 @@ cudaError_t launch_simt_gemm(int dtype, int M, int N, int K, const void* A, bool
                              cudaStream_t stream);
 
 // fp32 contraction on the tensor cores, each operand as three bf16 parts (split_gemm.cu).  The caller
-// provides the parts: launch_split3 makes those of up to kMaxSplitJobs matrices in one launch, and the
-// gate / dH epilogues write those of H / dG (EpiParams::H3, G3).
+// provides the parts: launch_split3 makes those of up to kMaxSplitJobs matrices in one launch.
+// An fp32 matrix as the sum of three bf16 ones: [3][rows, cols], row pitch a multiple of 8 elements.
+struct Parts {
+  void* base = nullptr;
+  int rows = 0, cols = 0, pitch = 0;
+};
+inline size_t parts_bytes(size_t rows, size_t cols) { return align_up(3 * rows * ((cols + 7) / 8 * 8) * 2, 256); }
 struct SplitJob { const float* src; Parts parts; };
 constexpr int kMaxSplitJobs = 6;
 cudaError_t launch_split3(const SplitJob* jobs, int n, cudaStream_t stream);
