@@ -215,8 +215,9 @@ __device__ __forceinline__ float ld_shared_cluster_f32(uint32_t cluster_addr) {
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
   return v;
 }
-__device__ __forceinline__ void ld_shared_cluster_f32x2(uint32_t cluster_addr, float& a, float& b) {
-  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(a), "=f"(b) : "r"(cluster_addr) : "memory");
+__device__ __forceinline__ void ld_shared_cluster_f32x4(uint32_t cluster_addr, float (&v)[4]) {
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(cluster_addr) : "memory");
 }
 __device__ __forceinline__ int ld_shared_cluster_s32(uint32_t cluster_addr) {
   int v;

@@ -9,7 +9,7 @@
 // tiles leaves most SMs without work.  Here the contraction is cut along k over the CTAs (pairs) of a
 // cluster until every SM streams an equal share of W; the CTAs leave their fp32 sums in shared memory,
 // and each adds one share of the batch over the cluster in ascending k and runs the epilogue on it,
-// pairs of neighbouring features per thread, so that table rows, G, H and y move in whole 128-byte lines.
+// four neighbouring features per thread, so that table rows, G, H and y move in whole 128-byte lines.
 //
 // Bound: streaming W (3.6 TB/s from a cold memory with all SMs loading, and at most 70 - 98 GB/s into one
 // SM), on top of a chain of launch, first loads, last MMA, exchange and epilogue of some 5 us per kernel.
@@ -161,19 +161,19 @@ stream_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     ptx::grid_dependency_wait();
     ptx::grid_launch_dependents();
     const int et = threadIdx.x - 64;
-    // final stage: features f, f + 1 of the tokens first, first + step, ... of this CTA's share
-    const int f = f0 + (et & 63) * 2, first = slice + ksplit * (et >> 6), step = ksplit * (kEpiThreads / 64);
+    // final stage: features f .. f + 3 of the tokens first, first + step, ... of this CTA's share
+    const int f = f0 + (et & 31) * 4, first = slice + ksplit * (et >> 5), step = ksplit * (kEpiThreads / 32);
     const bool f_ok = f < F;
-    // Sixteen 8-byte reads of other CTAs' sums are in flight per thread: those of 8 tokens from 2 CTAs, or
-    // of 4 tokens from 4 CTAs at a time.
-    const int batch = ksplit <= 2 ? 8 : 4;
-    uint32_t e[8];
-    auto request = [&](int t0) {      // table-row pairs of the next tokens
+    // Eight 16-byte reads of the CTAs' sums are in flight per thread: those of 4 tokens from 2 CTAs, or of 2
+    // tokens from 4 CTAs at a time.
+    const int batch = ksplit <= 2 ? 4 : 2;
+    uint2 e[4];
+    auto request = [&](int t0) {      // table-row pieces of the next tokens
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < 4; ++i) {
         const int t = t0 + i * step;
         if (KIND == kEpiGate && f_ok && i < batch && t < T)
-          e[i] = __ldg(reinterpret_cast<const uint32_t*>(static_cast<const __nv_bfloat16*>(ep.E) + static_cast<size_t>(s_ids[t]) * F + f));
+          e[i] = __ldg(reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(ep.E) + static_cast<size_t>(s_ids[t]) * F + f));
       }
     };
     if (KIND == kEpiGate) {
@@ -212,53 +212,60 @@ stream_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     // Every epilogue thread of the cluster meets here, also after a timeout (the other warps: below).
     if (clustered) ptx::cluster_sync(); else asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
     if (ok && f_ok) {
-      const uint32_t sums = base + 8u * (et & 63);
+      const uint32_t sums = base + 16u * (et & 31);
       // (Rolled up on purpose: this runs once, and a body unrolled over the tokens took 8300 cycles to fetch.)
       auto finish = [&](auto tokens, auto ctas) {
         constexpr int TB = decltype(tokens)::value, KB = decltype(ctas)::value;
 #pragma unroll 1
         for (int t0 = first; t0 < T; t0 += TB * step) {
-          uint32_t cur[TB];
-          float a0[TB], a1[TB];
+          uint2 cur[TB];
+          float a[TB][4];
 #pragma unroll
-          for (int i = 0; i < TB; ++i) { cur[i] = e[i]; a0[i] = 0.0f; a1[i] = 0.0f; }
+          for (int i = 0; i < TB; ++i) { cur[i] = e[i]; a[i][0] = a[i][1] = a[i][2] = a[i][3] = 0.0f; }
           if (t0 + TB * step < T) request(t0 + TB * step);
 #pragma unroll 1
           for (int k0 = 0; k0 < ksplit; k0 += KB) {
-            float p0[KB][TB], p1[KB][TB];
+            float p[KB][TB][4];
 #pragma unroll
             for (int k = 0; k < KB; ++k) {
               const uint32_t src = sums + 4u * BM * t0;
               const uint32_t at = clustered ? ptx::mapa(src, min(k0 + k, ksplit - 1) * CTAS + rank) : src;
 #pragma unroll
               for (int i = 0; i < TB; ++i) {
-                p0[k][i] = p1[k][i] = 0.0f;
-                if (k0 + k < ksplit && t0 + i * step < T) ptx::ld_shared_cluster_f32x2(at + 4u * BM * i * step, p0[k][i], p1[k][i]);
+                p[k][i][0] = p[k][i][1] = p[k][i][2] = p[k][i][3] = 0.0f;
+                if (k0 + k < ksplit && t0 + i * step < T) ptx::ld_shared_cluster_f32x4(at + 4u * BM * i * step, p[k][i]);
               }
             }
 #pragma unroll
             for (int k = 0; k < KB; ++k)
 #pragma unroll
-              for (int i = 0; i < TB; ++i) { a0[i] += p0[k][i]; a1[i] += p1[k][i]; }
+              for (int i = 0; i < TB; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) a[i][j] += p[k][i][j];
           }
 #pragma unroll
           for (int i = 0; i < TB; ++i) {
             const int t = t0 + i * step;
             if (t < T) {
               const size_t o = static_cast<size_t>(t) * F + f;
+              const uint2 acc = make_uint2(pack_bf16(a[i][0], a[i][1]), pack_bf16(a[i][2], a[i][3]));
               if (KIND == kEpiGate) {
-                const float u0 = __uint_as_float(cur[i] << 16), u1 = __uint_as_float(cur[i] & 0xFFFF0000u);
-                *reinterpret_cast<uint32_t*>(static_cast<__nv_bfloat16*>(ep.H) + o) =
-                    pack_bf16(a0[i] * fast_sigmoid(a0[i]) * u0, a1[i] * fast_sigmoid(a1[i]) * u1);
-                if (ep.G) *reinterpret_cast<uint32_t*>(static_cast<__nv_bfloat16*>(ep.G) + o) = pack_bf16(a0[i], a1[i]);
+                const float u[4] = {__uint_as_float(cur[i].x << 16), __uint_as_float(cur[i].x & 0xFFFF0000u),
+                                    __uint_as_float(cur[i].y << 16), __uint_as_float(cur[i].y & 0xFFFF0000u)};
+                float h[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) h[j] = a[i][j] * fast_sigmoid(a[i][j]) * u[j];
+                *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(ep.H) + o) =
+                    make_uint2(pack_bf16(h[0], h[1]), pack_bf16(h[2], h[3]));
+                if (ep.G) *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(ep.G) + o) = acc;
               } else {
-                *reinterpret_cast<uint32_t*>(static_cast<__nv_bfloat16*>(ep.out) + o) = pack_bf16(a0[i], a1[i]);
+                *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(ep.out) + o) = acc;
               }
             }
           }
         }
       };
-      if (batch == 8) finish(Int<8>{}, Int<2>{}); else finish(Int<4>{}, Int<4>{});
+      if (batch == 4) finish(Int<4>{}, Int<2>{}); else finish(Int<2>{}, Int<4>{});
     }
     __syncwarp();
   }
