@@ -564,7 +564,8 @@ Plan make_plan(int M1, int N1, int M2, int N2, int K) {
     const long long tiles = tile_count(M1, N1, BM * ctas, 64 * ctas) + tile_count(M2, N2, BM * ctas, 64 * ctas);
     for (int sp = 1; sp * ctas <= 8; sp *= 2) {
       if (sp > 1 && (tiles * sp > slots || k_blocks < 2 * sp)) break;
-      const double rounds = static_cast<double>((tiles * sp + slots - 1) / slots);
+      const int at_once = clusters_at_once(ctas * sp);
+      const double rounds = static_cast<double>((tiles + at_once - 1) / at_once);
       const double cost = rounds * ((k_blocks + sp - 1) / sp * 1750.0) + 3000.0 + (sp > 1 ? 2500.0 : 0.0);
       if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = {pair, sp}; }
     }

@@ -181,6 +181,7 @@ cudaError_t launch_shard_route(int n_max, int T, int G, const int32_t* unique_id
 cudaError_t launch_selftest_wait(int32_t* status, long long limit_cycles, int arrive, cudaStream_t stream);
 
 int device_sm_count();
+int clusters_at_once(int size);   // clusters of size (1 .. 8) CTAs that run together, one CTA per SM
 
 // Function attributes (shared-memory size, preferred split) are per device: `done` is a
 // per-call-site table that remembers on which devices `set()` has already succeeded.

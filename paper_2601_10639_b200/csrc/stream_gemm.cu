@@ -314,36 +314,6 @@ bool encode_operand(CUtensorMap* map, const void* ptr, int rows, int cols, int b
 constexpr int kMaxSmem = 232448;
 int smem_budget(int n_pad) { return n_pad <= 128 ? 113 * 1024 : kMaxSmem; }
 
-// Clusters of `size` CTAs that run at once with one CTA per SM (an SM left over in a GPC is no help to a
-// cluster that needs more of them: 15 clusters of 8, not 18).  Asked once per device and size.
-int max_clusters(int size) {
-  static int cached[64][9] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return device_sm_count() / size;
-  if (cached[dev][size] == 0) {
-    int n = 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(device_sm_count() / size * size));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kMaxSmem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = static_cast<unsigned>(size);
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    auto kern = stream_gemm_kernel<kEpiStore, 1>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
-      cudaGetLastError();
-      n = device_sm_count() / size;
-    }
-    cached[dev][size] = n;
-  }
-  return cached[dev][size];
-}
-
 // Single CTAs or pairs, and CTAs along k.  What a CTA must load sets the pace: its k range times 128 rows
 // of W and its rows of X (half of the batch in a pair), times the rounds its clusters take.  Narrow
 // batches get no more CTAs than there are SMs, though two fit one: the second place is a cluster's that
@@ -357,7 +327,7 @@ Plan make_plan(int T, int F, int K) {
     const int tiles = (F + BM * ctas - 1) / (BM * ctas), n_pad = (T + 16 * ctas - 1) / (16 * ctas) * (16 * ctas);
     for (int sp = 1; sp * ctas <= 8; ++sp) {
       if (sp > 1 && (k_blocks < 2 * sp || static_cast<long long>(tiles) * ctas * sp > slots)) break;
-      const int at_once = n_pad <= 128 ? slots / (ctas * sp) : max_clusters(ctas * sp);
+      const int at_once = n_pad <= 128 ? slots / (ctas * sp) : clusters_at_once(ctas * sp);
       const long long rounds = (tiles + at_once - 1) / at_once;
       const long long rows = rounds * ((k_blocks + sp - 1) / sp) * (BM + n_pad / ctas);
       if (best.rows == 0 || rows < best.rows) best = {ctas, sp, n_pad, rows};
@@ -409,6 +379,36 @@ cudaError_t launch_inst(const void* X, const void* W, int T, int F, int K, const
 }
 
 }  // namespace
+
+// Clusters of `size` CTAs that run at once with one CTA per SM (an SM left over in a GPC is no help to a
+// cluster that needs more of them: 15 clusters of 8, not 18).  Asked once per device and size.
+int clusters_at_once(int size) {
+  static int cached[64][9] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return device_sm_count() / size;
+  if (cached[dev][size] == 0) {
+    int n = 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(device_sm_count() / size * size));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kMaxSmem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(size);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    auto kern = stream_gemm_kernel<kEpiStore, 1>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+      cudaGetLastError();
+      n = device_sm_count() / size;
+    }
+    cached[dev][size] = n;
+  }
+  return cached[dev][size];
+}
 
 cudaError_t launch_stream_gemm(int T, int F, int K, const void* X, const void* W, EpiKind kind, const EpiParams& ep,
                                cudaStream_t stream) {
