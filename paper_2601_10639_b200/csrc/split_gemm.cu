@@ -12,10 +12,14 @@
 // Precision.  The tensor core does not round its fp32 accumulation to nearest, so long chains on it
 // drift.  Each 64-wide k block is therefore a sum of its own in tensor memory: the five small terms
 // first, the four x0 y0 instructions last, so that no more than four truncations act on a number of
-// the block sum's size; the block sums are added in fp32 registers, rounded to nearest.  A result
-// that is not finite (an input near the top of the range or not finite: its parts then hold infinities
-// of both signs) or below 2^-98 (third parts below 2^-133 are lost, an error of up to K 2^-134 times
-// the other operand) is computed again from the fp32 operands as one chain of FMAs in ascending k.
+// the block sum's size; the block sums are added in fp32 registers, rounded to nearest.
+//
+// Range.  The parts are those of 2^24 x.  They are multiples of x's last bit, at least 2^-149, so no part is
+// below 2^-125: none is lost or subnormal, however small x is and however large its partner.  (Parts of x itself
+// lose their last bits below 2^-110, all of them below 2^-134: 1e-38 against 1e10 was off by 6e-3, 1e-41
+// against 1e12 gave zero.)  The sums are 2^48 times the result and a power of two changes no rounding.  A result
+// that is not finite (sums beyond the range, infinite parts) is computed again from the fp32 operands as one
+// chain of FMAs in ascending k.
 //
 // The parts come from split3_kernel: one launch for the operands of a call, one for H or dG once they are
 // there.  (Written by the epilogue that makes H or dG instead, 16 bytes per row and instruction, they cost it
@@ -72,12 +76,16 @@ struct Smem {
 };
 
 // ---- the three parts ------------------------------------------------------------------------
+constexpr float kScale = 16777216.0f;                       // 2^24, of every operand
+constexpr float kUnscale = 1.0f / 281474976710656.0f;       // 2^-48, of the sums of their products
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&h);
 }
-// Two fp32 values -> the packed pairs of their first, second and third parts.
+// Two fp32 values -> the packed pairs of the first, second and third parts of kScale times them.
 __device__ __forceinline__ void split_pair(float a, float b, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
+  a *= kScale;
+  b *= kScale;
   p0 = pack2(a, b);
   const float ra = a - __uint_as_float(p0 << 16), rb = b - __uint_as_float(p0 & 0xFFFF0000u);
   p1 = pack2(ra, rb);
@@ -146,13 +154,8 @@ struct Product {
   bool wide = false;             // 32-byte accesses are legal in every [., N] matrix of the epilogue
 };
 
-// Results that the parts cannot carry: not finite, or so small that the third parts of the inputs fell
-// below bf16's smallest number.  Zero is what it is.
-__device__ __forceinline__ bool needs_chain(float v) {
-  const uint32_t u = __float_as_uint(v) & 0x7FFFFFFFu;
-  constexpr uint32_t kTiny = 29u << 23;   // 2^-98
-  return u - kTiny > 0x7F7FFFFFu - kTiny && u != 0;
-}
+// Results that the parts cannot carry: not finite.
+__device__ __forceinline__ bool needs_chain(float v) { return (__float_as_uint(v) & 0x7FFFFFFFu) > 0x7F7FFFFFu; }
 // The plain chain of FMAs for them; a[i] is column n + i of row m.  (A NaN stays one, so the chain ends
 // there.)
 template <bool A_MN, bool B_MN>
@@ -459,7 +462,7 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
           for (int n = n0; n < min(n0 + kCols, pr.N); n += 8) {
             float a8[8], e8[8], g8[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) { a8[i] = acc[i]; e8[i] = e[i]; g8[i] = g[i]; }
+            for (int i = 0; i < 8; ++i) { a8[i] = acc[i] * kUnscale; e8[i] = e[i]; g8[i] = g[i]; }
             load_operands<KIND>(ep, pr, m, n + 8, min(n0 + kCols, pr.N) - n - 8, id, e, g);
             redo_in_fp32<A_MN, B_MN>(pr, K, m, n, pr.N - n, a8);
             epilogue8<KIND>(ep, pr, m, n, pr.N - n, a8, e8, g8);
@@ -501,6 +504,8 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
 #pragma unroll
             for (int i = 0; i < 8; ++i) a8[i] += v[i];
           }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) a8[i] *= kUnscale;
           redo_in_fp32<A_MN, B_MN>(pr, K, m, n, end - n, a8);
           epilogue8<KIND>(ep, pr, m, n, end - n, a8, e8, g8);
         }
