@@ -227,6 +227,16 @@ __device__ __forceinline__ int ld_shared_cluster_s32(uint32_t cluster_addr) {
 __device__ __forceinline__ void st_shared_cluster_v2(uint32_t cluster_addr, int a, int b) {
   asm volatile("st.shared::cluster.v2.s32 [%0], {%1, %2};" ::"r"(cluster_addr), "r"(a), "r"(b) : "memory");
 }
+// Barrier `id` over `threads` threads of the CTA (whole warps); ..._or: whether `v` holds for any of them.
+__device__ __forceinline__ void named_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ bool named_sync_or(int id, int threads, bool v) {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %3, 0;\n\tbar.red.or.pred q, %1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+               : "=r"(r) : "r"(id), "r"(threads), "r"(static_cast<uint32_t>(v)) : "memory");
+  return r != 0;
+}
 // Barrier over all threads of all CTAs of the cluster.
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");

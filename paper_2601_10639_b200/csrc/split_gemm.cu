@@ -17,9 +17,15 @@
 // Range.  The parts are those of 2^24 x.  They are multiples of x's last bit, at least 2^-149, so no part is
 // below 2^-125: none is lost or subnormal, however small x is and however large its partner.  (Parts of x itself
 // lose their last bits below 2^-110, all of them below 2^-134: 1e-38 against 1e10 was off by 6e-3, 1e-41
-// against 1e12 gave zero.)  The sums are 2^48 times the result and a power of two changes no rounding.  A result
-// that is not finite (sums beyond the range, infinite parts) is computed again from the fp32 operands as one
-// chain of FMAs in ascending k.
+// against 1e12 gave zero.)  The sums are 2^48 times the result and a power of two changes no rounding.  Operands
+// below 2^24 cannot bring them to 2^128 at any K.  A launch with an operand that holds anything else (a value of
+// 2^24 or more, an infinity, a NaN) leaves its sums and computes every output as a chain of FMAs in ascending k, as the
+// FMA kernel does (fma_tiles, below).  split3_kernel, which sees every element, leaves a word per block of its
+// grid that says so; nothing has to be cleared, and the accumulating warps read the words while the first operands
+// arrive.  (Redoing just the results that came out infinite, by the thread that holds them and inside the pipeline,
+// took one chain of K loads after another: a backward pass over 2048 positions, 512 x 1024, with one infinity in
+// dy 19.7 ms, against 0.55 so, 0.68 on the FMA kernels and 0.10 without the infinity; the pipeline's own waits
+// would have run out beyond some 1e5 positions.)
 //
 // The parts come from split3_kernel: one launch for the operands of a call, one for H or dG once they are
 // there.  (Written by the epilogue that makes H or dG instead, 16 bytes per row and instruction, they cost it
@@ -54,7 +60,8 @@ namespace {
 constexpr int BM = 128;
 constexpr int BK = 64;
 constexpr int kAccWarps = 8;
-constexpr int kThreads = 32 * (2 + kAccWarps);
+constexpr int kAccThreads = 32 * kAccWarps;
+constexpr int kThreads = 64 + kAccThreads;
 constexpr long long kWaitLimitCycles = 2000000000ll;  // ~1 s at boost clock
 
 template <int BN, int CTAS>
@@ -78,6 +85,7 @@ struct Smem {
 // ---- the three parts ------------------------------------------------------------------------
 constexpr float kScale = 16777216.0f;                       // 2^24, of every operand
 constexpr float kUnscale = 1.0f / 281474976710656.0f;       // 2^-48, of the sums of their products
+constexpr uint32_t kLimitBits = 0x4B800000u;                // 2^24: the parts carry what is below
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&h);
@@ -97,10 +105,12 @@ struct SplitList {
   int first_block[kMaxSplitJobs + 1];   // blocks [first_block[i], first_block[i + 1]) work on job i
   int n;
 };
-constexpr int kSplitThreads = 256, kSplitPieces = 2;   // 8-column pieces per thread
+constexpr int kSplitPieces = 2;                        // 8-column pieces per thread
+constexpr int kSplitThreads = kPiecesPerWord / kSplitPieces;
 
 // fp32 [rows, cols] -> bf16 [3][rows, pitch], pitch = cols rounded up to 8.  Bound by memory: 4 bytes
-// read and 6 written per element, every access a whole vector of its row.
+// read and 6 written per element, every access a whole vector of its row.  A block also leaves the word that
+// says whether it met a value the parts cannot carry.
 __global__ void __launch_bounds__(kSplitThreads) split3_kernel(const __grid_constant__ SplitList list) {
   ptx::grid_dependency_wait();
   ptx::grid_launch_dependents();
@@ -112,6 +122,7 @@ __global__ void __launch_bounds__(kSplitThreads) split3_kernel(const __grid_cons
   const long long p0 = static_cast<long long>(blockIdx.x - list.first_block[j]) * (kSplitThreads * kSplitPieces) + threadIdx.x;
   const size_t plane = static_cast<size_t>(job.parts.rows) * job.parts.pitch;
   float4 v[kSplitPieces][2];
+  uint32_t top = 0;                        // largest magnitude of this thread's values (their bits)
 #pragma unroll
   for (int i = 0; i < kSplitPieces; ++i) {
     const long long p = p0 + i * kSplitThreads;
@@ -132,6 +143,10 @@ __global__ void __launch_bounds__(kSplitThreads) split3_kernel(const __grid_cons
   for (int i = 0; i < kSplitPieces; ++i) {
     const long long p = p0 + i * kSplitThreads;
     if (p >= pieces) continue;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      top = max(max(top, max(__float_as_uint(v[i][h].x) & 0x7FFFFFFFu, __float_as_uint(v[i][h].y) & 0x7FFFFFFFu)),
+                max(__float_as_uint(v[i][h].z) & 0x7FFFFFFFu, __float_as_uint(v[i][h].w) & 0x7FFFFFFFu));
     uint4 o[3];
     split_pair(v[i][0].x, v[i][0].y, o[0].x, o[1].x, o[2].x);
     split_pair(v[i][0].z, v[i][0].w, o[0].y, o[1].y, o[2].y);
@@ -141,42 +156,23 @@ __global__ void __launch_bounds__(kSplitThreads) split3_kernel(const __grid_cons
 #pragma unroll
     for (int s = 0; s < 3; ++s) *reinterpret_cast<uint4*>(dst + s * plane) = o[s];
   }
+  const int beyond = __syncthreads_or(top >= kLimitBits);
+  if (threadIdx.x == 0) job.parts.words()[blockIdx.x - list.first_block[j]] = beyond;
 }
 
 // ---- epilogue ---------------------------------------------------------------------------------
 // One product of the launch.  A second one with the same K and layouts may ride along (plain stores
 // only); its tiles are numbered after the first one's.
 struct Product {
-  const float* A = nullptr;      // the fp32 operands, for results that the parts cannot carry
+  const float* A = nullptr;      // the fp32 operands, for values that the parts cannot carry
   const float* B = nullptr;
+  const uint32_t* a_words = nullptr;   // not zero: a block of A's (B's) parts met such a value
+  const uint32_t* b_words = nullptr;
+  int a_n = 0, b_n = 0;
   float* out = nullptr;
   int M = 0, N = 0;
   bool wide = false;             // 32-byte accesses are legal in every [., N] matrix of the epilogue
 };
-
-// Results that the parts cannot carry: not finite.
-__device__ __forceinline__ bool needs_chain(float v) { return (__float_as_uint(v) & 0x7FFFFFFFu) > 0x7F7FFFFFu; }
-// The plain chain of FMAs for them; a[i] is column n + i of row m.  (A NaN stays one, so the chain ends
-// there.)
-template <bool A_MN, bool B_MN>
-__device__ __forceinline__ void redo_in_fp32(const Product& pr, int K, int m, int n, int have, float (&a)[8]) {
-  uint32_t marked = 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-    if (needs_chain(a[i]) && i < have) marked |= 1u << i;
-  while (marked != 0) {
-    const int i = __ffs(marked) - 1;
-    marked &= marked - 1;
-    float acc = 0.0f;
-#pragma unroll 1
-    for (int k = 0; k < K && acc == acc; ++k)
-      acc = fmaf(A_MN ? pr.A[static_cast<size_t>(k) * pr.M + m] : pr.A[static_cast<size_t>(m) * K + k],
-                 B_MN ? pr.B[static_cast<size_t>(k) * pr.N + n + i] : pr.B[static_cast<size_t>(n + i) * K + k], acc);
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (j == i) a[j] = acc;
-  }
-}
 
 // Eight consecutive values of a row; WIDE: the row pitch and the base are multiples of 32 bytes.
 // have: how many of them exist (a multiple of 4, at most 8).  Plain loads: kEpiAdd may overwrite its addend.
@@ -252,6 +248,77 @@ __device__ __forceinline__ int table_row(const EpiParams& ep, int m) {
     id = id < 0 ? 0 : ep.V - 1;
   }
   return id;
+}
+
+// ---- operands that the parts cannot carry --------------------------------------------------------
+__device__ __forceinline__ bool any_word(const uint32_t* words, int n, int et) {
+  uint32_t any = 0;
+#pragma unroll 4
+  for (int i = et; i < n; i += kAccThreads) any |= words[i];
+  return any != 0;
+}
+// The outputs of the whole launch by the accumulating warps of its CTAs, 64 x 64 at a time: one chain of FMAs
+// in ascending k for each.  (These CTAs hold their SM alone, so the next k step's operands are requested before the
+// present one's FMAs.)  smem: the operand ring, free by now.
+template <bool A_MN, bool B_MN, int KIND>
+__device__ __noinline__ void fma_tiles(const EpiParams& ep, const Product& p1, const Product& p2, int K, float* smem, int et) {
+  constexpr int FT = 64, FK = 16, kPitch = FT + 4;
+  const int tx = et & 15, ty = et >> 4;
+  const int tm1 = (p1.M + FT - 1) / FT, tm2 = (p2.M + FT - 1) / FT;
+  const long long tiles1 = static_cast<long long>(tm1) * ((p1.N + FT - 1) / FT);
+  const long long tiles = tiles1 + static_cast<long long>(tm2) * ((p2.N + FT - 1) / FT);
+  int buf = 0;
+  for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const bool second = KIND == kEpiStore && tile >= tiles1;
+    const Product& pr = second ? p2 : p1;
+    const long long tt = second ? tile - tiles1 : tile;
+    const int tm = second ? tm2 : tm1, m0 = static_cast<int>(tt % tm) * FT, n0 = static_cast<int>(tt / tm) * FT;
+    float acc[4][4] = {}, ra[4], rb[4];
+    auto fetch = [&](int k0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int idx = et + i * kAccThreads;
+        const int am = A_MN ? idx % FT : idx / FK, ak = k0 + (A_MN ? idx / FT : idx % FK);
+        const int bn = B_MN ? idx % FT : idx / FK, bk = k0 + (B_MN ? idx / FT : idx % FK);
+        ra[i] = m0 + am < pr.M && ak < K
+                    ? (A_MN ? pr.A[static_cast<size_t>(ak) * pr.M + m0 + am] : pr.A[static_cast<size_t>(m0 + am) * K + ak]) : 0.0f;
+        rb[i] = n0 + bn < pr.N && bk < K
+                    ? (B_MN ? pr.B[static_cast<size_t>(bk) * pr.N + n0 + bn] : pr.B[static_cast<size_t>(n0 + bn) * K + bk]) : 0.0f;
+      }
+    };
+    fetch(0);
+    for (int k0 = 0; k0 < K; k0 += FK, buf ^= 1) {
+      float* As = smem + buf * (2 * FK * kPitch);
+      float* Bs = As + FK * kPitch;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int idx = et + i * kAccThreads;
+        As[(A_MN ? idx / FT : idx % FK) * kPitch + (A_MN ? idx % FT : idx / FK)] = ra[i];
+        Bs[(B_MN ? idx / FT : idx % FK) * kPitch + (B_MN ? idx % FT : idx / FK)] = rb[i];
+      }
+      ptx::named_sync(1, kAccThreads);      // (nobody still reads the other buffer's last step behind this one)
+      if (k0 + FK < K) fetch(k0 + FK);
+#pragma unroll
+      for (int kk = 0; kk < FK; ++kk) {
+        const float4 a = *reinterpret_cast<const float4*>(As + kk * kPitch + ty * 4);
+        const float4 b = *reinterpret_cast<const float4*>(Bs + kk * kPitch + tx * 4);
+        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+      }
+    }
+    const int n = n0 + tx * 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int m = m0 + ty * 4 + i;
+      if (m >= pr.M || n >= pr.N) continue;
+      float a8[8] = {acc[i][0], acc[i][1], acc[i][2], acc[i][3]}, e8[8] = {}, g8[8] = {};
+      load_operands<KIND>(ep, pr, m, n, 4, KIND != kEpiStore ? table_row<KIND>(ep, m) : 0, e8, g8);
+      epilogue8<KIND>(ep, pr, m, n, 4, a8, e8, g8);
+    }
+  }
 }
 
 // ---- the contraction ----------------------------------------------------------------------------
@@ -414,6 +481,10 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
     int buf = 0; uint32_t bph = 0;
     float acc[kCols], e[8], g[8];
     const int share = kCols / ksplit;       // columns of a tile that this thread finishes
+    const int et = threadIdx.x - 64;
+    bool beyond = any_word(p1.a_words, p1.a_n, et) || any_word(p1.b_words, p1.b_n, et);
+    if (KIND == kEpiStore && tiles2 > 0) beyond = beyond || any_word(p2.a_words, p2.a_n, et) || any_word(p2.b_words, p2.b_n, et);
+    beyond = ptx::named_sync_or(1, kAccThreads, beyond);
     int id = 0;
     for (int tile = tile0; ok && tile < num_tiles; tile += tile_step) {
       const bool second = KIND == kEpiStore && tile >= tiles1;
@@ -457,14 +528,13 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
       if (ksplit == 1) {
         // Eight columns at a time in a rolled loop, the sums moving down: unrolled over the columns this is
         // some 3000 instructions that a launch has to fetch first (layer of 256 rows: 79.5 -> 75 us rolled).
-        if (m < pr.M) {
+        if (m < pr.M && !beyond) {
 #pragma unroll 1
           for (int n = n0; n < min(n0 + kCols, pr.N); n += 8) {
             float a8[8], e8[8], g8[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) { a8[i] = acc[i] * kUnscale; e8[i] = e[i]; g8[i] = g[i]; }
             load_operands<KIND>(ep, pr, m, n + 8, min(n0 + kCols, pr.N) - n - 8, id, e, g);
-            redo_in_fp32<A_MN, B_MN>(pr, K, m, n, pr.N - n, a8);
             epilogue8<KIND>(ep, pr, m, n, pr.N - n, a8, e8, g8);
 #pragma unroll
             for (int i = 0; i + 8 < kCols; ++i) acc[i] = acc[i + 8];
@@ -486,7 +556,7 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
       const Product& pr = second ? p2 : p1;
       const int tt = second ? tile0 - tiles1 : tile0, tm = second ? tiles_m2 : tiles_m1;
       const int m = tt % tm * TM + rank * BM + r, n0 = tt / tm * BN + half * kCols + slice * share;
-      if (ok && m < pr.M) {
+      if (ok && m < pr.M && !beyond) {
         const uint32_t mine = base + 4u * (static_cast<uint32_t>(half * kCols + slice * share) * BM + r);
         const int end = min(n0 + share, pr.N);
 #pragma unroll 1
@@ -506,12 +576,15 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
           }
 #pragma unroll
           for (int i = 0; i < 8; ++i) a8[i] *= kUnscale;
-          redo_in_fp32<A_MN, B_MN>(pr, K, m, n, end - n, a8);
           epilogue8<KIND>(ep, pr, m, n, end - n, a8, e8, g8);
         }
       }
       __syncwarp();
     }
+    // Every copy into this CTA's ring and every MMA on it is complete (as above), and no CTA of the cluster reads it.
+    if (beyond && !ptx::named_sync_or(1, kAccThreads, !ok))
+      fma_tiles<A_MN, B_MN, KIND>(ep, p1, p2, K, reinterpret_cast<float*>(base_ptr), et);
+    __syncwarp();
   }
 
   if (ksplit > 1 && warp < 2) { __syncwarp(); ptx::cluster_sync(); }   // (the other warps': above)
@@ -600,7 +673,10 @@ cudaError_t launch_inst(const SplitProduct& a, const SplitProduct& b, int K, int
   auto a32 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 31u) == 0; };
   for (int i = 0; i < 2; ++i) {
     const bool wide = src[i]->N % 8 == 0 && a32(src[i]->out) && a32(ep.E) && a32(ep.Gin) && a32(ep.H) && a32(ep.G);
-    p[i] = {src[i]->A, src[i]->B, src[i]->out, src[i]->M, src[i]->N, wide};
+    p[i].A = src[i]->A; p[i].B = src[i]->B;
+    p[i].a_words = src[i]->A3.words(); p[i].a_n = src[i]->A3.n_words();
+    p[i].b_words = src[i]->B3.words(); p[i].b_n = src[i]->B3.n_words();
+    p[i].out = src[i]->out; p[i].M = src[i]->M; p[i].N = src[i]->N; p[i].wide = wide;
   }
   const long long tiles = tile_count(a.M, a.N, BM * CTAS, BN) + tile_count(b.M, b.N, BM * CTAS, BN);
   const int slots = device_sm_count() / CTAS;
@@ -643,8 +719,7 @@ cudaError_t launch_split3(const SplitJob* jobs, int n, cudaStream_t stream) {
     if (list.n == kMaxSplitJobs || p.cols % 4) return cudaErrorNotSupported;
     list.job[list.n] = jobs[i];
     list.first_block[list.n++] = static_cast<int>(blocks);
-    const long long pieces = static_cast<long long>(p.rows) * (p.pitch / 8), per_block = kSplitThreads * kSplitPieces;
-    blocks += (pieces + per_block - 1) / per_block;
+    blocks += p.n_words();
   }
   if (list.n == 0) return cudaSuccess;
   if (blocks > 0x7fffffffll) return cudaErrorNotSupported;

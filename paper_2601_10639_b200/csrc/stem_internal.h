@@ -73,12 +73,22 @@ cudaError_t launch_simt_gemm(int dtype, int M, int N, int K, const void* A, bool
 
 // fp32 contraction on the tensor cores, each operand as three bf16 parts (split_gemm.cu).  The caller
 // provides the parts: launch_split3 makes those of up to kMaxSplitJobs matrices in one launch.
-// An fp32 matrix as the sum of three bf16 ones: [3][rows, cols], row pitch a multiple of 8 elements.
+// An fp32 matrix as the sum of three bf16 ones: [3][rows, cols], row pitch a multiple of 8 elements; behind
+// them a word for every kPiecesPerWord 8-column pieces, not zero where a value cannot be carried so.
+constexpr int kPiecesPerWord = 512;
+inline size_t part_words(size_t rows, size_t pitch) { return (rows * (pitch / 8) + kPiecesPerWord - 1) / kPiecesPerWord; }
 struct Parts {
   void* base = nullptr;
   int rows = 0, cols = 0, pitch = 0;
+  int n_words() const { return static_cast<int>(part_words(rows, pitch)); }
+  __host__ __device__ uint32_t* words() const {
+    return reinterpret_cast<uint32_t*>(static_cast<char*>(base) + static_cast<size_t>(6) * rows * pitch);
+  }
 };
-inline size_t parts_bytes(size_t rows, size_t cols) { return align_up(3 * rows * ((cols + 7) / 8 * 8) * 2, 256); }
+inline size_t parts_bytes(size_t rows, size_t cols) {
+  const size_t pitch = (cols + 7) / 8 * 8;
+  return align_up(6 * rows * pitch + 4 * part_words(rows, pitch), 256);
+}
 struct SplitJob { const float* src; Parts parts; };
 constexpr int kMaxSplitJobs = 6;
 cudaError_t launch_split3(const SplitJob* jobs, int n, cudaStream_t stream);
