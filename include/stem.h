@@ -93,7 +93,11 @@ int stem_version(void);
 const char* stem_status_string(int code);
 
 /* Bytes of workspace that any call with this shape needs (the maximum over calls).
- * The first 256 bytes of a workspace hold the status word. */
+ * The first 256 bytes of a workspace hold the status word.
+ * fp32: the tensor-core contractions keep three bf16 parts of every operand in the workspace, which makes
+ * it some 3.5 times as large.  Where memory is short, ask with STEM_FLAG_SIMT in the flags: calls (with
+ * or without the flag) that are given that smaller workspace run on the FMA kernels, with the same
+ * results within fp32 rounding, several times slower.  stem_step_arena_bytes() likewise. */
 int stem_workspace_bytes(const stem_shape_t* shape, size_t* bytes /*host, out*/);
 
 /* Clear the status word.  Call once after allocating a workspace (and to re-arm it

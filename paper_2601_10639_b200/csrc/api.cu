@@ -118,6 +118,7 @@ struct WsLayout {
   size_t h_off, h_bytes;     // forward: H when the caller keeps none
   size_t du_off, dg_off, tf_bytes, part_off, part_bytes, sk_off, sk_bytes;
   size_t x3_off, dy3_off, wg3_off, wd3_off, h3_off, dg3_off;   // fp32: the operands' bf16 parts
+  size_t min_total;          // what every call needs: fp32 contractions run on the FMA kernels without the parts
   size_t total;
 };
 
@@ -139,7 +140,8 @@ WsLayout ws_layout(const stem_shape_t* s) {
   size_t m = w.dedup_off + w.dedup_bytes;
   if (w.h_off + w.h_bytes > m) m = w.h_off + w.h_bytes;
   if (w.sk_off + w.sk_bytes > m) m = w.sk_off + w.sk_bytes;
-  if (s->dtype == STEM_DTYPE_FP32) {
+  w.min_total = align_up(m, 256);
+  if (s->dtype == STEM_DTYPE_FP32 && !(s->flags & STEM_FLAG_SIMT)) {
     m = align_up(m, 1024);
     const size_t td = parts_bytes(s->T, s->d_model), fd = parts_bytes(s->d_ff, s->d_model), df = parts_bytes(s->d_model, s->d_ff),
                  tf3 = parts_bytes(s->T, s->d_ff);
@@ -159,9 +161,10 @@ bool use_tc(const stem_shape_t* s) {
   return s->dtype == STEM_DTYPE_BF16 && !(s->flags & STEM_FLAG_SIMT);
 }
 
-// fp32 on the tensor cores (three bf16 parts per operand)
-bool use_split(const stem_shape_t* s) {
-  return s->dtype == STEM_DTYPE_FP32 && !(s->flags & STEM_FLAG_SIMT) && is_sm100();
+// fp32 on the tensor cores (three bf16 parts per operand), where the workspace has room for the parts: they
+// make it about 3.5 times as large (2048 positions, 1024 x 2816: 181 against 52 MB).
+bool use_split(const stem_shape_t* s, const WsLayout& w, size_t ws_bytes) {
+  return s->dtype == STEM_DTYPE_FP32 && !(s->flags & STEM_FLAG_SIMT) && ws_bytes >= w.total && is_sm100();
 }
 
 // An fp32 operand and where its parts lie in the workspace.
@@ -263,7 +266,7 @@ int stem_dedup_ids(const stem_shape_t* shape, const int32_t* ids, int32_t* uniqu
   if (!unique_ids || !n_unique || !perm || !seg_offsets || !ws || !aligned16(ws)) return STEM_ERR_INVALID_ARG;
   if (shape->T > 0 && !ids) return STEM_ERR_INVALID_ARG;
   const WsLayout w = ws_layout(shape);
-  if (ws_bytes < w.total) return STEM_ERR_WORKSPACE_TOO_SMALL;
+  if (ws_bytes < w.min_total) return STEM_ERR_WORKSPACE_TOO_SMALL;
   ProfScope prof("dedup", static_cast<cudaStream_t>(stream));
   cudaError_t e = launch_dedup(shape->T, shape->V, ids, unique_ids, n_unique, inverse, perm, seg_offsets,
                                static_cast<char*>(ws) + w.dedup_off, status_of(ws), static_cast<cudaStream_t>(stream));
@@ -281,7 +284,7 @@ int stem_ffn_forward(const stem_shape_t* shape, const void* x, const int32_t* id
       !aligned16(G_save) || !aligned16(H_save))
     return STEM_ERR_INVALID_ARG;
   const WsLayout w = ws_layout(shape);
-  if (ws_bytes < w.total) return STEM_ERR_WORKSPACE_TOO_SMALL;
+  if (ws_bytes < w.min_total) return STEM_ERR_WORKSPACE_TOO_SMALL;
   if (use_tc(shape) && !is_sm100()) return STEM_ERR_UNSUPPORTED_ARCH;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int T = shape->T, d = shape->d_model, F = shape->d_ff;
@@ -290,7 +293,7 @@ int stem_ffn_forward(const stem_shape_t* shape, const void* x, const int32_t* id
   EpiParams gate;
   gate.ids = ids; gate.E = E; gate.V = shape->V; gate.H = H; gate.G = G_save; gate.status = status_of(ws);
   cudaError_t e;
-  if (use_split(shape)) {
+  if (use_split(shape, w, ws_bytes)) {
     const Operand x3 = operand(ws, w.x3_off, x, T, d), wg3 = operand(ws, w.wg3_off, W_gate, F, d),
                   wd3 = operand(ws, w.wd3_off, W_down, d, F), h3 = operand(ws, w.h3_off, H, T, F);
     {
@@ -355,7 +358,7 @@ static int ffn_backward(const stem_shape_t* shape, const void* dy, const void* x
       !aligned16(dW_down) || !aligned16(dE_rows))
     return STEM_ERR_INVALID_ARG;
   const WsLayout w = ws_layout(shape);
-  if (ws_bytes < w.total) return STEM_ERR_WORKSPACE_TOO_SMALL;
+  if (ws_bytes < w.min_total) return STEM_ERR_WORKSPACE_TOO_SMALL;
   if (use_tc(shape) && !is_sm100()) return STEM_ERR_UNSUPPORTED_ARCH;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int T = shape->T, d = shape->d_model, F = shape->d_ff;
@@ -369,7 +372,7 @@ static int ffn_backward(const stem_shape_t* shape, const void* dy, const void* x
   EpiParams dh;
   dh.ids = ids; dh.E = E; dh.V = shape->V; dh.H = dU; dh.G = dG; dh.Gin = G_save; dh.status = status_of(ws);
   cudaError_t e;
-  const bool split = use_split(shape);
+  const bool split = use_split(shape, w, ws_bytes);
   const Operand dy3 = operand(ws, w.dy3_off, dy, T, d), x3 = operand(ws, w.x3_off, x, T, d),
                 wg3 = operand(ws, w.wg3_off, W_gate, F, d), wd3 = operand(ws, w.wd3_off, W_down, d, F),
                 h3 = operand(ws, w.h3_off, H_save, T, F), dg3 = operand(ws, w.dg3_off, dG, T, F);
@@ -509,7 +512,7 @@ int stem_reduce_rows(const stem_shape_t* shape, const void* rows_in, const int32
   if (!rows_in || !perm || !seg_offsets || !n_unique || !rows_out || !aligned16(rows_in) || !aligned16(rows_out))
     return STEM_ERR_INVALID_ARG;
   const WsLayout w = ws_layout(shape);
-  if (ws_bytes < w.total) return STEM_ERR_WORKSPACE_TOO_SMALL;
+  if (ws_bytes < w.min_total) return STEM_ERR_WORKSPACE_TOO_SMALL;
   ProfScope prof("reduce_rows", static_cast<cudaStream_t>(stream));
   cudaError_t e = launch_segreduce(shape->T, shape->d_ff, shape->grad_dtype, shape->grad_dtype, rows_in, perm,
                                    seg_offsets, n_unique, rows_out, static_cast<char*>(ws) + w.part_off,
@@ -529,7 +532,7 @@ int stem_dagger_forward(const stem_shape_t* shape, const void* x, const int32_t*
       !aligned16(G_save) || !aligned16(H_save) || !aligned16(U_save))
     return STEM_ERR_INVALID_ARG;
   const WsLayout w = ws_layout(shape);
-  if (ws_bytes < w.total) return STEM_ERR_WORKSPACE_TOO_SMALL;
+  if (ws_bytes < w.min_total) return STEM_ERR_WORKSPACE_TOO_SMALL;
   if (use_tc(shape) && !is_sm100()) return STEM_ERR_UNSUPPORTED_ARCH;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int T = shape->T, d = shape->d_model, F = shape->d_ff;
@@ -548,7 +551,7 @@ int stem_dagger_forward(const stem_shape_t* shape, const void* x, const int32_t*
     e = launch_tc_gemm_dagger(T, F, d, x, W_gate, W_up, du, st);
     if (e != cudaSuccess) return cuda_fail(e);
   } else {
-    const bool split = use_split(shape);
+    const bool split = use_split(shape, w, ws_bytes);
     const Operand x3 = operand(ws, w.x3_off, x, T, d), wg3 = operand(ws, w.wg3_off, W_gate, F, d),
                   wu3 = operand(ws, w.wd3_off, W_up, F, d);
     if (split) {
@@ -573,7 +576,7 @@ int stem_dagger_forward(const stem_shape_t* shape, const void* x, const int32_t*
     }
     if (e != cudaSuccess) return cuda_fail(e);
   }
-  if (use_split(shape)) {   // W_down's parts take the place of W_up's
+  if (use_split(shape, w, ws_bytes)) {   // W_down's parts take the place of W_up's
     const Operand h3 = operand(ws, w.h3_off, H, T, F), wd3 = operand(ws, w.wd3_off, W_down, d, F);
     EpiParams down;
     down.out = y; down.status = status_of(ws);
@@ -608,7 +611,7 @@ int stem_dagger_backward(const stem_shape_t* shape, const void* dy, const void* 
       !aligned16(dW_up) || !aligned16(dW_down) || !aligned16(dE_rows))
     return STEM_ERR_INVALID_ARG;
   const WsLayout w = ws_layout(shape);
-  if (ws_bytes < w.total) return STEM_ERR_WORKSPACE_TOO_SMALL;
+  if (ws_bytes < w.min_total) return STEM_ERR_WORKSPACE_TOO_SMALL;
   if (use_tc(shape) && !is_sm100()) return STEM_ERR_UNSUPPORTED_ARCH;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int T = shape->T, d = shape->d_model, F = shape->d_ff;
@@ -617,7 +620,7 @@ int stem_dagger_backward(const stem_shape_t* shape, const void* dy, const void* 
   void* dU = base + w.du_off;
   void* dG = base + w.dg_off;
   cudaError_t e;
-  const bool split = use_split(shape);
+  const bool split = use_split(shape, w, ws_bytes);
   const Operand dy3 = operand(ws, w.dy3_off, dy, T, d), x3 = operand(ws, w.x3_off, x, T, d),
                 wg3 = operand(ws, w.wg3_off, W_gate, F, d), wd3 = operand(ws, w.wd3_off, W_down, d, F),
                 h3 = operand(ws, w.h3_off, H_save, T, F), dg3 = operand(ws, w.dg3_off, dG, T, F);
@@ -870,13 +873,13 @@ namespace {
 struct Arena {
   size_t ws, ws_bytes, x[2], dy[2], ids[2], y[2], dx[2], n_u[2], G, H, inverse, perm, seg, total;
 };
-Arena arena_layout(const stem_shape_t* s) {
+Arena arena_layout(const stem_shape_t* s, size_t ws_bytes) {
   Arena a{};
   const size_t T = s->T, td = align_up(T * s->d_model * elem_bytes(s->dtype), 256),
                tf = align_up(T * s->d_ff * elem_bytes(s->dtype), 256), ti = align_up((T + 1) * 4, 256);
   const size_t R = static_cast<size_t>(s->T < s->V ? s->T : s->V);
   size_t o = 0;
-  a.ws = o; a.ws_bytes = ws_layout(s).total; o += a.ws_bytes;
+  a.ws = o; a.ws_bytes = ws_bytes; o += a.ws_bytes;
   for (int k = 0; k < 2; ++k) {
     a.x[k] = o; o += td;  a.dy[k] = o; o += td;  a.ids[k] = o; o += ti;
     a.y[k] = o; o += td;  a.dx[k] = o; o += td;
@@ -924,7 +927,7 @@ cudaError_t pipe_get(StepPipe** out) {
 int stem_step_arena_bytes(const stem_shape_t* shape, size_t* bytes) {
   if (!bytes) return STEM_ERR_INVALID_ARG;
   if (int rc = check_shape(shape)) return rc;
-  *bytes = arena_layout(shape).total;
+  *bytes = arena_layout(shape, ws_layout(shape).total).total;
   return STEM_OK;
 }
 
@@ -936,7 +939,9 @@ int stem_ffn_step_host(const stem_shape_t* shape, const void* host_x, const int3
   if (!arena || !aligned16(arena)) return STEM_ERR_INVALID_ARG;
   if (shape->T == 0) return STEM_OK;
   if (!host_x || !host_ids || !host_dy || !host_y || !host_dx || !unique_ids || !n_unique) return STEM_ERR_INVALID_ARG;
-  const Arena a = arena_layout(shape);
+  const WsLayout w = ws_layout(shape);
+  Arena a = arena_layout(shape, w.total);
+  if (arena_bytes < a.total) a = arena_layout(shape, w.min_total);
   if (arena_bytes < a.total) return STEM_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   std::lock_guard<std::mutex> lock(g_pipe_mutex);
