@@ -131,6 +131,7 @@ stream_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     if (lane == 0 && rank == 0) {
       const uint32_t idesc = ptx::make_idesc_bf16(BM * CTAS, n_pad, false, false);
       const uint16_t pair_mask = static_cast<uint16_t>(3u << leader);
+      ptx::grid_dependency_wait();   // nothing is read here, but the limit of the waits below must not run before
       int s = 0; uint32_t ph = 0;
       for (int kb = kb0; kb < kb1; ++kb) {
         if (!ptx::mbar_wait_bounded(full_bar(s), ph, abort_flag, kWaitLimitCycles)) {
