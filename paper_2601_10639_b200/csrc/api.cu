@@ -191,9 +191,10 @@ SplitProduct split_product(const Operand& a, const Operand& b, void* out, int M,
   p.M = M; p.N = N;
   return p;
 }
-cudaError_t split_gemm(int M, int N, int K, const Operand& a, bool a_mn, const Operand& b, bool b_mn, EpiKind kind,
-                       const EpiParams& ep, cudaStream_t st) {
-  return launch_split_gemm(split_product(a, b, ep.out, M, N), SplitProduct{}, K, a_mn, b_mn, kind, ep, st);
+cudaError_t split_gemm(const stem_shape_t* s, int M, int N, int K, const Operand& a, bool a_mn, const Operand& b, bool b_mn,
+                       EpiKind kind, const EpiParams& ep, cudaStream_t st) {
+  return launch_split_gemm(split_product(a, b, ep.out, M, N), SplitProduct{}, K, a_mn, b_mn, kind, ep,
+                           !(s->flags & STEM_FLAG_SINGLE_CTA), st);
 }
 
 cudaError_t gemm(const stem_shape_t* s, int M, int N, int K, const void* A, bool a_mn, const void* B,
@@ -303,7 +304,7 @@ int stem_ffn_forward(const stem_shape_t* shape, const void* x, const int32_t* id
     if (e != cudaSuccess) return cuda_fail(e);
     {
       ProfScope prof("gate_gemm", st);
-      e = split_gemm(T, F, d, x3, false, wg3, false, kEpiGate, gate, st);
+      e = split_gemm(shape, T, F, d, x3, false, wg3, false, kEpiGate, gate, st);
     }
     if (e != cudaSuccess) return cuda_fail(e);
     EpiParams down;
@@ -314,7 +315,7 @@ int stem_ffn_forward(const stem_shape_t* shape, const void* x, const int32_t* id
     }
     if (e != cudaSuccess) return cuda_fail(e);
     ProfScope prof("down_gemm", st);
-    e = split_gemm(T, d, F, h3, false, wd3, false, kEpiStore, down, st);
+    e = split_gemm(shape, T, d, F, h3, false, wd3, false, kEpiStore, down, st);
     return e == cudaSuccess ? STEM_OK : cuda_fail(e);
   }
   // a few rows: the weight matrices stream through once
@@ -386,7 +387,7 @@ static int ffn_backward(const stem_shape_t* shape, const void* dy, const void* x
     if (e != cudaSuccess) return cuda_fail(e);
     {
       ProfScope prof("dh_gemm", st);
-      e = split_gemm(T, F, d, dy3, false, wd3, true, kEpiDH, dh, st);
+      e = split_gemm(shape, T, F, d, dy3, false, wd3, true, kEpiDH, dh, st);
     }
     if (e != cudaSuccess) return cuda_fail(e);
     ProfScope prof("split_operands", st);
@@ -400,7 +401,7 @@ static int ffn_backward(const stem_shape_t* shape, const void* dy, const void* x
     EpiParams p; p.out = dx; p.out_fp32 = shape->dtype == STEM_DTYPE_FP32; p.status = status_of(ws);
     p.sk_scratch = base + w.sk_off; p.sk_bytes = w.sk_bytes;
     ProfScope prof("dx_gemm", st);
-    return split ? split_gemm(T, d, F, dg3, false, wg3, true, kEpiStore, p, st)
+    return split ? split_gemm(shape, T, d, F, dg3, false, wg3, true, kEpiStore, p, st)
                  : gemm(shape, T, d, F, dG, false, W_gate, true, kEpiStore, p, st);
   };
   if (dx && dx_done) {
@@ -421,7 +422,8 @@ static int ffn_backward(const stem_shape_t* shape, const void* dy, const void* x
   if (split && (dW_down || dW_gate)) {
     const SplitProduct down = split_product(dy3, h3, dW_down, d, F), gate = split_product(dg3, x3, dW_gate, F, d);
     ProfScope prof("dw_pair_gemm", st);
-    e = launch_split_gemm(dW_down ? down : gate, dW_down && dW_gate ? gate : SplitProduct{}, T, true, true, kEpiStore, gp, st);
+    e = launch_split_gemm(dW_down ? down : gate, dW_down && dW_gate ? gate : SplitProduct{}, T, true, true, kEpiStore, gp,
+                          !(shape->flags & STEM_FLAG_SINGLE_CTA), st);
     if (e != cudaSuccess) return cuda_fail(e);
   } else if (dW_down && dW_gate && use_tc(shape)) {
     // dW_down[i,j] = sum_t dy[t,i] H[t,j] and dW_gate[j,k] = sum_t dG[t,j] x[t,k] in ONE launch: both
@@ -563,7 +565,7 @@ int stem_dagger_forward(const stem_shape_t* shape, const void* x, const int32_t*
       EpiParams up;
       up.ids = ids; up.E = E; up.V = shape->V; up.H = U_save; up.status = status_of(ws);
       ProfScope prof("up_gemm", st);
-      e = split ? split_gemm(T, F, d, x3, false, wu3, false, kEpiAdd, up, st)
+      e = split ? split_gemm(shape, T, F, d, x3, false, wu3, false, kEpiAdd, up, st)
                 : gemm(shape, T, F, d, x, false, W_up, false, kEpiAdd, up, st);
     }
     if (e != cudaSuccess) return cuda_fail(e);
@@ -571,7 +573,7 @@ int stem_dagger_forward(const stem_shape_t* shape, const void* x, const int32_t*
       EpiParams gate;
       gate.ids = nullptr; gate.E = U_save; gate.V = T; gate.H = H; gate.G = G_save; gate.status = status_of(ws);
       ProfScope prof("gate_gemm", st);
-      e = split ? split_gemm(T, F, d, x3, false, wg3, false, kEpiGate, gate, st)
+      e = split ? split_gemm(shape, T, F, d, x3, false, wg3, false, kEpiGate, gate, st)
                 : gemm(shape, T, F, d, x, false, W_gate, false, kEpiGate, gate, st);
     }
     if (e != cudaSuccess) return cuda_fail(e);
@@ -582,7 +584,7 @@ int stem_dagger_forward(const stem_shape_t* shape, const void* x, const int32_t*
     down.out = y; down.status = status_of(ws);
     ProfScope prof("down_gemm", st);
     e = split3({wd3, h3}, st);
-    if (e == cudaSuccess) e = split_gemm(T, d, F, h3, false, wd3, false, kEpiStore, down, st);
+    if (e == cudaSuccess) e = split_gemm(shape, T, d, F, h3, false, wd3, false, kEpiStore, down, st);
     return e == cudaSuccess ? STEM_OK : cuda_fail(e);
   }
   EpiParams down;
@@ -633,7 +635,7 @@ int stem_dagger_backward(const stem_shape_t* shape, const void* dy, const void* 
     if (split) {
       Operand none{};
       e = split3({dy3, wd3, x3, wg3, dW_down ? h3 : none}, st);
-      if (e == cudaSuccess) e = split_gemm(T, F, d, dy3, false, wd3, true, kEpiDH, dh, st);
+      if (e == cudaSuccess) e = split_gemm(shape, T, F, d, dy3, false, wd3, true, kEpiDH, dh, st);
     } else {
       e = gemm(shape, T, F, d, dy, false, W_down, true, kEpiDH, dh, st);
     }
@@ -643,7 +645,7 @@ int stem_dagger_backward(const stem_shape_t* shape, const void* dy, const void* 
     EpiParams p; p.out = out; p.status = status_of(ws);
     p.accumulate = (shape->flags & STEM_FLAG_ACCUM_GRADS) != 0;
     ProfScope prof(name, st);
-    return split_gemm(M, N, T, A, true, Bm, true, kEpiStore, p, st);
+    return split_gemm(shape, M, N, T, A, true, Bm, true, kEpiStore, p, st);
   };
   auto grad = [&](const char* name, void* out, int M, int N, const void* A, const void* Bm) {
     EpiParams p; p.out = out; p.out_fp32 = grad_fp32; p.status = status_of(ws);
@@ -686,13 +688,13 @@ int stem_dagger_backward(const stem_shape_t* shape, const void* dy, const void* 
     EpiParams p; p.out = dx; p.out_fp32 = shape->dtype == STEM_DTYPE_FP32; p.status = status_of(ws);
     {
       ProfScope prof("dx_gemm", st);
-      e = split ? split_gemm(T, d, F, dg3, false, wg3, true, kEpiStore, p, st)
+      e = split ? split_gemm(shape, T, d, F, dg3, false, wg3, true, kEpiStore, p, st)
                 : gemm(shape, T, d, F, dG, false, W_gate, true, kEpiStore, p, st);
     }
     if (e != cudaSuccess) return cuda_fail(e);
     EpiParams a; a.ids = nullptr; a.E = dx; a.V = T; a.H = dx; a.status = status_of(ws);
     ProfScope prof("dx_up_gemm", st);
-    e = split ? split_gemm(T, d, F, du3, false, wu3, true, kEpiAdd, a, st)
+    e = split ? split_gemm(shape, T, d, F, du3, false, wu3, true, kEpiAdd, a, st)
               : gemm(shape, T, d, F, dU, false, W_up, true, kEpiAdd, a, st);
     if (e != cudaSuccess) return cuda_fail(e);
   }

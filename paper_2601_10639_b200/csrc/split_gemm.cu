@@ -633,11 +633,12 @@ bool encode_parts(CUtensorMap* map, const Parts& p, int box_rows) {
 // costs.  A cluster has at most 8 CTAs, and a slice at least 2 blocks.
 struct Plan { bool pair; int ksplit; };
 long long tile_count(int M, int N, int tm, int bn) { return static_cast<long long>((M + tm - 1) / tm) * ((N + bn - 1) / bn); }
-Plan make_plan(int M1, int N1, int M2, int N2, int K) {
+Plan make_plan(int M1, int N1, int M2, int N2, int K, bool pairs) {
   const int k_blocks = (K + BK - 1) / BK;
-  Plan best{true, 1};
+  Plan best{pairs, 1};
   double best_cost = 0.0;
   for (bool pair : {true, false}) {
+    if (pair && !pairs) continue;
     const int ctas = pair ? 2 : 1, slots = device_sm_count() / ctas;
     const long long tiles = tile_count(M1, N1, BM * ctas, 64 * ctas) + tile_count(M2, N2, BM * ctas, 64 * ctas);
     for (int sp = 1; sp * ctas <= 8; sp *= 2) {
@@ -701,8 +702,9 @@ cudaError_t launch_inst(const SplitProduct& a, const SplitProduct& b, int K, int
 }
 
 template <bool A_MN, bool B_MN, int KIND>
-cudaError_t launch_planned(const SplitProduct& a, const SplitProduct& b, int K, const EpiParams& ep, cudaStream_t stream) {
-  const Plan pl = make_plan(a.M, a.N, b.M, b.N, K);
+cudaError_t launch_planned(const SplitProduct& a, const SplitProduct& b, int K, const EpiParams& ep, bool pairs,
+                           cudaStream_t stream) {
+  const Plan pl = make_plan(a.M, a.N, b.M, b.N, K, pairs);
   if (pl.pair) return launch_inst<A_MN, B_MN, KIND, 2>(a, b, K, pl.ksplit, ep, stream);
   return launch_inst<A_MN, B_MN, KIND, 1>(a, b, K, pl.ksplit, ep, stream);
 }
@@ -739,21 +741,21 @@ cudaError_t launch_split3(const SplitJob* jobs, int n, cudaStream_t stream) {
 }
 
 cudaError_t launch_split_gemm(const SplitProduct& p, const SplitProduct& second, int K, bool a_mn, bool b_mn, EpiKind kind,
-                              const EpiParams& ep, cudaStream_t stream) {
+                              const EpiParams& ep, bool pairs, cudaStream_t stream) {
   if (p.M <= 0 || p.N <= 0) return cudaSuccess;
   if (K <= 0 || (p.N % 4) || (second.N % 4)) return cudaErrorNotSupported;
   // the layer's call sites: gate, up (K,K)  down (K,K,store)  dH, dx (K,MN)  dW_* (MN,MN,store)
   if (second.M > 0 && !(a_mn && b_mn && kind == kEpiStore)) return cudaErrorNotSupported;
   if (!a_mn && !b_mn) {
-    if (kind == kEpiGate) return launch_planned<false, false, kEpiGate>(p, second, K, ep, stream);
-    if (kind == kEpiAdd) return launch_planned<false, false, kEpiAdd>(p, second, K, ep, stream);
-    if (kind == kEpiStore) return launch_planned<false, false, kEpiStore>(p, second, K, ep, stream);
+    if (kind == kEpiGate) return launch_planned<false, false, kEpiGate>(p, second, K, ep, pairs, stream);
+    if (kind == kEpiAdd) return launch_planned<false, false, kEpiAdd>(p, second, K, ep, pairs, stream);
+    if (kind == kEpiStore) return launch_planned<false, false, kEpiStore>(p, second, K, ep, pairs, stream);
   } else if (!a_mn && b_mn) {
-    if (kind == kEpiDH) return launch_planned<false, true, kEpiDH>(p, second, K, ep, stream);
-    if (kind == kEpiAdd) return launch_planned<false, true, kEpiAdd>(p, second, K, ep, stream);
-    if (kind == kEpiStore) return launch_planned<false, true, kEpiStore>(p, second, K, ep, stream);
+    if (kind == kEpiDH) return launch_planned<false, true, kEpiDH>(p, second, K, ep, pairs, stream);
+    if (kind == kEpiAdd) return launch_planned<false, true, kEpiAdd>(p, second, K, ep, pairs, stream);
+    if (kind == kEpiStore) return launch_planned<false, true, kEpiStore>(p, second, K, ep, pairs, stream);
   } else if (a_mn && b_mn) {
-    if (kind == kEpiStore) return launch_planned<true, true, kEpiStore>(p, second, K, ep, stream);
+    if (kind == kEpiStore) return launch_planned<true, true, kEpiStore>(p, second, K, ep, pairs, stream);
   }
   return cudaErrorNotSupported;
 }

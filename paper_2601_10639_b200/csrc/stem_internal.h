@@ -94,7 +94,7 @@ constexpr int kMaxSplitJobs = 6;
 cudaError_t launch_split3(const SplitJob* jobs, int n, cudaStream_t stream);
 // Same contraction, layouts and epilogues as below with fp32 storage; extents that are contiguous in
 // memory are multiples of 4, else cudaErrorNotSupported.  `second` (M == 0: none) rides in the same
-// launch: token-contracted plain stores only.
+// launch: token-contracted plain stores only.  pairs: CTA pairs may be used where they are the faster form.
 struct SplitProduct {
   const float* A = nullptr;
   const float* B = nullptr;
@@ -103,7 +103,7 @@ struct SplitProduct {
   int M = 0, N = 0;
 };
 cudaError_t launch_split_gemm(const SplitProduct& p, const SplitProduct& second, int K, bool a_mn, bool b_mn, EpiKind kind,
-                              const EpiParams& ep, cudaStream_t stream);
+                              const EpiParams& ep, bool pairs, cudaStream_t stream);
 
 // tcgen05 / TMEM / TMA kernels, bf16 inputs.  Returns cudaErrorNotSupported when the
 // shape cannot be described to TMA (the caller decides what to do).
