@@ -899,7 +899,7 @@ cudaError_t launch_tc_gemm(int M, int N, int K, const void* A, bool a_mn, const 
   // TMA needs 16-byte row pitches (the contiguous extent of each operand a multiple of 8
   // elements); the epilogue stores 8 columns at a time.
   if (K <= 0 || (N % 8) || ((a_mn ? M : K) % 8) || ((b_mn ? N : K) % 8)) return cudaErrorNotSupported;
-  // layer call sites: gate (K,K,gate)  down (K,K,store)  dH (K,MN,dh)  dx (K,MN,store)
+  // layer call sites: gate (K,K,gate)  dagger's up (K,K,add)  down (K,K,store)  dH (K,MN,dh)  dx (K,MN,store)
   //                   dW_down / dW_gate (MN,MN,store); the plain-GEMM entry adds (MN,K,store)
   if (!a_mn && !b_mn) {
     if (kind == kEpiGate) return launch_ctas<false, false, kEpiGate>(A, B, M, N, K, ep, pair, stream);
@@ -907,7 +907,6 @@ cudaError_t launch_tc_gemm(int M, int N, int K, const void* A, bool a_mn, const 
     if (kind == kEpiStore) return launch_ctas<false, false, kEpiStore>(A, B, M, N, K, ep, pair, stream);
   } else if (!a_mn && b_mn) {
     if (kind == kEpiDH) return launch_ctas<false, true, kEpiDH>(A, B, M, N, K, ep, pair, stream);
-    if (kind == kEpiAdd) return launch_ctas<false, true, kEpiAdd>(A, B, M, N, K, ep, pair, stream);
     if (kind == kEpiStore) return launch_ctas<false, true, kEpiStore>(A, B, M, N, K, ep, pair, stream);
   } else if (a_mn && b_mn) {
     if (kind == kEpiStore) return launch_ctas<true, true, kEpiStore>(A, B, M, N, K, ep, pair, stream);
