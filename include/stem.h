@@ -365,6 +365,9 @@ int stem_reduce_rows(const stem_shape_t* shape, const void* rows_in, const int32
  * been called and `stream` synchronised (flush makes `stream` wait for every outstanding
  * output copy; it is cheap and may be called after every step at the price of the
  * overlap).  Calls on one device are serialised by a lock; use one arena at a time.
+ * A thread whose last flush on the device followed a single call is taken to wait for every call's
+ * outputs: its first call after a flush makes dx ahead of the table and weight gradients, so that its copy runs under them.
+ * The results do not depend on the order.
  */
 int stem_step_arena_bytes(const stem_shape_t* shape, size_t* bytes /*host, out*/);
 int stem_ffn_step_host(const stem_shape_t* shape, const void* host_x, const int32_t* host_ids,

@@ -900,14 +900,19 @@ struct StepPipe {
   cudaStream_t in = nullptr, out = nullptr;
   cudaEvent_t x_in[2], dy_in[2], y_done[2], dx_done[2], bwd_done[2], out_done[2];
   bool used[2] = {false, false};
-  int since_flush = 0;              // calls since the last flush
-  bool flush_each = false;          // the last flush came after a single call
   unsigned long long calls = 0;
 };
 std::mutex g_pipe_mutex;
 StepPipe g_pipe[64];
 
-cudaError_t pipe_get(StepPipe** out) {
+// How the calling thread flushes, per device.
+struct FlushHabit {
+  int since_flush = 0;              // calls since the last flush
+  bool flush_each = false;          // the last flush that had calls before it came after a single one
+};
+thread_local FlushHabit t_flush_habit[64];
+
+cudaError_t pipe_get(StepPipe** out, FlushHabit** habit) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -922,6 +927,7 @@ cudaError_t pipe_get(StepPipe** out) {
     p.ready = true;
   }
   *out = &p;
+  *habit = &t_flush_habit[dev];
   return cudaSuccess;
 }
 }  // namespace
@@ -948,17 +954,18 @@ int stem_ffn_step_host(const stem_shape_t* shape, const void* host_x, const int3
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   std::lock_guard<std::mutex> lock(g_pipe_mutex);
   StepPipe* pp = nullptr;
-  cudaError_t e = pipe_get(&pp);
+  FlushHabit* habit = nullptr;
+  cudaError_t e = pipe_get(&pp, &habit);
   if (e != cudaSuccess) return cuda_fail(e);
   StepPipe& p = *pp;
   const int k = static_cast<int>(p.calls++ & 1);   // slot of this call
-  // A caller that flushes after every call (as it did after the last one) waits for this call's outputs before its next one computes: dx is
-  // made first and leaves under the weight gradients.  Where calls follow one another without a flush, that
+  // A thread that flushes after every call (as it did after its last one) waits for this call's outputs before its
+  // next one computes: dx is made first and leaves under the weight gradients.  Where calls follow one another without a flush, that
   // would only crowd the two directions of the link.  Measured, 2048 x 8192, flush after every call / calls in a
   // row, dx last against dx first: 16384 positions 3796 / 2931 against 3448 / 2945 us, 9000: 2137 / 1635
   // against 1920 / 1700, 5000: 1220 / 930 against 1103 / 1015, 2500: 715 / 496 against 605 / 560.
-  const bool dx_first = p.flush_each && p.since_flush == 0;
-  ++p.since_flush;
+  const bool dx_first = habit->flush_each && habit->since_flush == 0;
+  ++habit->since_flush;
   char* base = static_cast<char*>(arena);
   const size_t td = static_cast<size_t>(shape->T) * shape->d_model * elem_bytes(shape->dtype);
   int32_t* ids = reinterpret_cast<int32_t*>(base + a.ids[k]);
@@ -1010,12 +1017,13 @@ int stem_ffn_step_host(const stem_shape_t* shape, const void* host_x, const int3
 int stem_ffn_step_host_flush(void* stream) {
   std::lock_guard<std::mutex> lock(g_pipe_mutex);
   StepPipe* pp = nullptr;
-  cudaError_t e = pipe_get(&pp);
+  FlushHabit* habit = nullptr;
+  cudaError_t e = pipe_get(&pp, &habit);
   if (e != cudaSuccess) return cuda_fail(e);
   for (int k = 0; k < 2; ++k)
     if (pp->used[k]) STEP_CUDA(cudaStreamWaitEvent(static_cast<cudaStream_t>(stream), pp->out_done[k], 0));
-  pp->flush_each = pp->since_flush == 1;
-  pp->since_flush = 0;
+  if (habit->since_flush > 0) habit->flush_each = habit->since_flush == 1;
+  habit->since_flush = 0;
 #undef STEP_CUDA
   return STEM_OK;
 }
