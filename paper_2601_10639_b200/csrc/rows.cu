@@ -16,14 +16,27 @@ namespace {
 
 constexpr int kThreads = 256;          // device-to-device gathers
 constexpr int kHostLinkCtas = 32;      // write-back
-// Row gathers across the link take twice as many: while a write-back fills the link's other direction, the
+// Row gathers across the link take up to twice as many: while a write-back fills the link's other direction, the
 // requests of 32 CTAs (0.5 MB in flight) brought 13 MB in 1208 us, alone in 430.  A layer of 8192 positions, three
 // host tables, forward and backward: 2799 us with 32 CTAs, 2268 with 64, 2340 with 96, 2450 with 128.
 constexpr int kHostGatherCtas = 64;
 constexpr int kHostLinkThreads = 128;
-// A decode step's rows are few and the step waits for them: one CTA per row, so that no row's chain of
-// id, slot, host read waits for another's.  (With 32 CTAs such chains were five rows long at 147 rows.)
-constexpr int kDecodeRows = 512;
+// Up to kFewRows rows no write-back is long enough to matter, and what CTAs ask for beyond kFewRowsBytes in
+// flight only takes from the forward pass beside it.  A forward layer with the next one's rows gathered beside
+// it, 32 / 64 / 512 CTAs, us: 2048 x 8192 (16 KB rows) 128 positions 42.3 / 45.3 / 48.4, 256: 63.1 / 69.1 / 83.1, 512: 98.0 /
+// 97.6 / 121.2; 1024 x 2816 (5.6 KB rows, a third of a CTA's requests) 256: 35.1 / 34.9 / 35.9, 512: 51.9 / 43.4 / 53.5.
+// With nothing beside it a gather of 256 such rows takes 54.6 / 44.5 / 44.5, of 16 KB rows 99 with any of them.
+constexpr int kFewRows = 512;
+constexpr int kFewRowsBytes = 512 * 1024;
+// With a hot set most rows come from the device, in between those that cross the link, and a decode step waits
+// for all of them: a CTA per row up to kHotRows rows, so that no row's chain of id, slot, host read waits for
+// another's.  A decode step (touch, dedup, gather, forward; 2048 cached rows), 32 / 64 / 512 CTAs, us: 2048 x 8192, 64
+// positions 31.1 / 29.8 / 29.7, 256: 60.7 / 55.8 / 54.0, 512: 92.7 / 86.3 / 80.6, 1024: 156 / 144 / 134, 2048: 248 / 230 /
+// 215; 1024 x 2816, 256: 39.0 / 33.9 / 33.1, 1024: 77.9 / 63.9 / 59.6.  The line is where this begins to cost more
+// beside another layer's contractions than it gives alone: a forward layer so, 2048 x 8192, 700 positions 80.9 /
+// 82.8 / 75.3, 1024: 99.9 / 106.3 / 108.2, 2048: 168 / 149 / 193, 8192: 606 / 542 / 783.
+constexpr int kHotRows = 1024;
+constexpr int kHotCtas = 512;
 
 __global__ void __launch_bounds__(kThreads)
 gather_rows_kernel(int max_rows, int V, int vec_per_row, const int32_t* __restrict__ ids,
@@ -178,7 +191,10 @@ cudaError_t launch_gather_rows(int max_rows, int V, size_t row_bytes, const int3
   const int lanes_per_row = vec < threads ? vec : threads;
   const int rows_per_cta = threads / lanes_per_row;
   int blocks = (max_rows + rows_per_cta - 1) / rows_per_cta;
-  const int cap = max_rows <= kDecodeRows ? kDecodeRows : kHostGatherCtas;
+  int cap = kHostGatherCtas;
+  if (hot_slot != nullptr && max_rows <= kHotRows) cap = kHotCtas;
+  else if (hot_slot == nullptr && max_rows <= kFewRows && row_bytes * kHostGatherCtas > kFewRowsBytes)
+    cap = row_bytes * kHostLinkCtas > kFewRowsBytes ? kHostLinkCtas : static_cast<int>(kFewRowsBytes / row_bytes);
   if (blocks > cap) blocks = cap;
   if (!table_on_host) {
     // a device table: flat copy, as many CTAs as the largest possible count needs, up to 8 per SM
