@@ -1,9 +1,10 @@
 """STEM-dagger backward on the tensor cores vs the CPU checker, where its launches can go wrong: the three weight
 gradients in one launch (tiles of three products, a split last round), dx as one contraction over two pairs of
-operands whose ragged 64-wide blocks do not line up, gradients left out, gradients accumulated."""
+operands whose ragged 64-wide blocks do not line up (whole, and cut along k), gradients left out, gradients accumulated."""
 import numpy as np
 import pytest
 import torch
+from torch.profiler import ProfilerActivity, profile
 
 from oracle import stem_oracle as O
 from paper_2601_10639_b200 import binding as B
@@ -33,15 +34,25 @@ def _run(T, d, F, flags, left_out=(), start=None):
                            b["seg_offsets"], b["n_unique"], out["dx"], out["dW_gate"], out["dW_up"], out["dW_down"],
                            out["dE_rows"], b["ws"])
     assert st.status() == B.OK
-    return inp, W_up, {k: v for k, v in out.items() if v is not None}
+    n = int(b["n_unique"].item())
+    return inp, W_up, {k: v[:n] if k == "dE_rows" else v for k, v in out.items() if v is not None}
 
 
 @pytest.mark.parametrize("flags", [0, B.FLAG_SINGLE_CTA], ids=["pair", "single"])
-@pytest.mark.parametrize("T,d,F", [(130, 72, 136), (300, 264, 520), (8200, 520, 1096)])
-def test_gradients(T, d, F, flags):
-    inp, W_up, got = _run(T, d, F, flags)
+# splits: launches whose last round is cut along k (and then finished by tail_fixup_kernel): the weight gradients of the
+# last but one size (few tiles, 8200 positions), dx of the last one (few tiles, 2 x 4104 deep, pieces on both
+# sides of the change of operands); the others save too little by it
+@pytest.mark.parametrize("T,d,F,splits", [(130, 72, 136, 0), (300, 264, 520, 0), (8200, 520, 1096, 0), (8200, 264, 520, 1),
+                                          (300, 264, 4104, 1)])
+def test_gradients(T, d, F, splits, flags):
+    with profile(activities=[ProfilerActivity.CUDA, ProfilerActivity.CPU]) as prof:
+        inp, W_up, got = _run(T, d, F, flags)
+        torch.cuda.synchronize()
+    ran = {e.key: e.count for e in prof.key_averages()}
+    assert sum(n for k, n in ran.items() if "tc_gemm_kernel" in k) == 6      # up, gate, down; dH, three gradients, dx
+    assert sum(n for k, n in ran.items() if "tail_fixup_kernel" in k) == splits, ran
     ref = O.dagger_backward(inp["dy"], inp["x"], inp["ids"], inp["W_gate"], W_up, inp["E"], inp["W_down"])
-    for k in ("dx", "dW_gate", "dW_up", "dW_down"):
+    for k in ("dx", "dW_gate", "dW_up", "dW_down", "dE_rows"):
         # a sum of few bf16-rounded terms can cancel to an entry far below them: the whole-tensor measures
         assert O.scaled_max_err(_np(got[k]), ref[k]) <= TOL_BF16 and O.rel_frobenius_err(_np(got[k]), ref[k]) <= 1e-2, k
 
@@ -52,8 +63,7 @@ def test_left_out_and_accumulated_gradients_agree_with_the_whole_call():
     for left_out in (("dW_up",), ("dW_down", "dx"), ("dW_gate", "dE_rows")):
         _, _, part = _run(T, d, F, 0, left_out)
         for k, v in part.items():
-            n = 0 if k == "dE_rows" else v.shape[0]
-            assert torch.equal(v[:n], whole[k][:n]), (left_out, k)
+            assert torch.equal(v, whole[k]), (left_out, k)
     _, _, acc = _run(T, d, F, B.FLAG_ACCUM_GRADS, start=0.5)
     for k in ("dW_gate", "dW_up", "dW_down"):
         assert (acc[k] - 0.5 - whole[k]).abs().max() <= 2e-6 * (0.5 + whole[k].abs().max()), k   # one fp32 addition
