@@ -16,7 +16,7 @@
 //
 // Range.  The parts are those of 2^24 x.  They are multiples of x's last bit, at least 2^-149, so no part is
 // below 2^-125: none is lost or subnormal, however small x is and however large its partner.  (Parts of x itself
-// lose their last bits below 2^-110, all of them below 2^-134: 1e-38 against 1e10 was off by 6e-3, 1e-41
+// lose their last bits below 2^-110, all of them below 2^-134: 1e-38 against 1e10 was off by 3e-3, 1e-41
 // against 1e12 gave zero.)  The sums are 2^48 times the result and a power of two changes no rounding.  Operands
 // below 2^24 cannot bring them to 2^128 at any K.  A launch with an operand that holds anything else (a value of
 // 2^24 or more, an infinity, a NaN) leaves its sums and computes every output as a chain of FMAs in ascending k, as the
@@ -32,8 +32,8 @@
 // 24 us of 109 at 2048 x 2816 where the launch costs 10.)  Splitting inside the contraction instead, on the way from
 // global to shared memory, converts every operand once per tile row or column that uses it and is bound
 // by that.  Measured, a layer's training step at 2048 positions, d_model 1024, d_ff 2816: 3600 us on the
-// FMA kernel, 787 us splitting inside, 494 us so (down, dx 62 us = 192 TFLOP/s each; gate 83, dH 94,
-// the weight gradients 125); at 256 positions, 256, 688: 237, 72 and 74 us.  Error against 64 bits:
+// FMA kernel, 787 us splitting inside, 519 us so (down, dx 62 us = 190 TFLOP/s each; gate 87, dH 102,
+// the weight gradients 126); at 256 positions, 256, 688: 238, 72 and 72 us.  Error against 64 bits:
 // 0.2 - 0.5 of the FMA kernel's for K >= 128, alike at K = 8.
 //
 // A tile is 128 * CTAS rows x BN columns.  CTAS = 2: a pair of CTAs shares each MMA (cta_group::2), each
@@ -42,9 +42,10 @@
 // pair) issues the 24 MMAs of a block, warps 2..9 add each finished block sum to their registers (one
 // row per thread, two warps per TMEM lane quarter, each half of the columns) and run the epilogue.
 //
-// Bound: shared-memory bandwidth and MMA rate nearly alike.  Per 64-wide block of a pair's tile each CTA
-// is written 72 KB and the MMAs read 144 KB of it, 1730 cycles at 128 bytes a clock, for 1536 cycles of
-// MMA.
+// Bound: a 64-wide block of a pair's tile takes 2100 - 2300 cycles (down at 22 to 176 blocks: 36 to 212 us at 1.965 GHz) for
+// 1536 of MMA.  Each CTA's shared memory is written 72 KB for it and read 6 KB by each of the 24 MMAs (128 rows of
+// A, 64 columns of B): 216 KB, 1730 cycles at 128 bytes a clock, so its bandwidth comes before the MMA rate; what the
+// other 400 - 600 cycles wait for is not known.
 //
 // A launch that would leave SMs idle is cut along k over the CTAs (pairs) of a cluster: each leaves its
 // sums in its own shared memory, and each then adds one share of the columns over the cluster in
@@ -628,8 +629,8 @@ bool encode_parts(CUtensorMap* map, const Parts& p, int box_rows) {
 }
 
 // Tile shape and k split.  The time of a launch is its rounds of tiles over the SMs times the k blocks of
-// a tile times a block's cost (1750 cycles for either shape, by shared-memory bytes; a pair's tile is
-// four times as large on twice the SMs), plus a tile's own latencies, plus what adding the slices
+// a tile times a block's cost (1750 cycles for either shape, by shared-memory bytes: a pair's
+// measured 2100 - 2300, but the plan only compares; a pair's tile is four times as large on twice the SMs), plus a tile's own latencies, plus what adding the slices
 // costs.  A cluster has at most 8 CTAs, and a slice at least 2 blocks.
 struct Plan { bool pair; int ksplit; };
 long long tile_count(int M, int N, int tm, int bn) { return static_cast<long long>((M + tm - 1) / tm) * ((N + bn - 1) / bn); }

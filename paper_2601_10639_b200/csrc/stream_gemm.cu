@@ -11,11 +11,12 @@
 // and each adds one share of the batch over the cluster in ascending k and runs the epilogue on it,
 // four neighbouring features per thread, so that table rows, G, H and y move in whole 128-byte lines.
 //
-// Bound: streaming W (3.6 TB/s from a cold memory with all SMs loading, and at most 70 - 98 GB/s into one
-// SM), on top of a chain of launch, first loads, last MMA, exchange and epilogue of some 5 us per kernel.
-// Measured, a forward pass (two of these kernels against two general ones), weights in L2 / not:
-//   d_model 2048, d_ff 8192   16 rows 32.4 -> 17.1 / 35.2 -> 20.8 us     128 rows 31.3 -> 26.0 us
-//   d_model 1024, d_ff 2816   16 rows 26.0 -> 12.1 us                    128 rows 27.0 -> 18.3 us
+// Bound: streaming W, on top of a chain of launch, first loads, last MMA, exchange and epilogue of some 5 us per
+// kernel.  33.5 MB of cold weights take 9.6 us, 3.5 TB/s over the kernel: 4.6 us of streaming at the memory's 7.3
+// TB/s and that chain.  (One SM draws at most 70 - 98 GB/s.)
+// Measured, a forward pass (two of these kernels against two general ones) replayed from a graph, weights in L2 / not:
+//   d_model 2048, d_ff 8192   16 rows 30.8 -> 14.9 / 32.5 -> 19.2 us     128 rows 29.8 -> 23.6 / 31.3 -> 28.0 us
+//   d_model 1024, d_ff 2816   16 rows 22.0 ->  9.3 / 23.0 -> 10.8 us     128 rows 22.9 -> 14.9 / 23.8 -> 16.5 us
 // Loading W before the kernel that writes X has finished gained nothing: the two then share the memory's
 // bandwidth (23.7 us against 21.2 with it left out, 16 rows, weights not in L2).
 #include <cuda.h>
@@ -427,13 +428,20 @@ cudaError_t launch_stream_gemm(int T, int F, int K, const void* X, const void* W
 }
 
 // Above 128 rows a CTA has no room for a second one beside it and the exchange (fp32 sums of the whole batch)
-// grows, so the lines depend on how much W there is to stream.  Measured, both forms of both kernels of a
-// forward pass, general / this one, 144, 192, 256 rows:
-//   2048 x 8192   31.7 / 25.7   33.0 / 27.4   34.0 / 32.9 us
-//   1800 x 6000   29.3 / 24.4   30.2 / 26.5   31.8 / 30.1
-//   1536 x 5000   24.5 / 22.5   27.3 / 25.0   28.4 / 28.7
-//   1024 x 2816   27.0 / 22.0   27.1 / 20.3   28.0 / 22.7, and 19.6, 20.5, 21.8 with only the second kernel so
-// (a plain store of a short k range per CTA: up to 3000 rows of operands, 6 blocks x 384 there).
+// grows, so the lines depend on how much W there is to stream.  Measured, a forward pass with both kernels general /
+// with both so / with only the second so, weights in L2, replayed from a graph, us at 144, 192, 256 rows:
+//   2048 x 8192   29.9 / 23.7 / 25.9   31.2 / 25.2 / 26.9   32.1 / 31.0 / 31.7
+//   1800 x 6000   27.8 / 22.2 / 24.4   28.6 / 24.2 / 25.8   30.0 / 27.8 / 28.1
+//   1536 x 5000   25.4 / 20.0 / 22.3   25.6 / 22.2 / 23.9   26.8 / 25.8 / 26.3
+//   1280 x 4096   29.1 / 17.1 / 18.6   29.2 / 18.9 / 19.7   30.1 / 21.8 / 21.5
+//   2048 x 2048   24.2 / 16.5 / 20.2   24.5 / 17.2 / 20.4   25.1 / 19.8 / 22.4
+//   1024 x 4096   27.9 / 16.6 / 17.3   28.1 / 18.0 / 18.4   28.7 / 20.6 / 20.0
+//   1024 x 2816   23.1 / 19.1 / 16.7   23.3 / 17.3 / 17.6   23.9 / 19.6 / 19.2
+//    768 x 2048   19.1 / 15.0 / 15.1   19.2 / 19.8 / 16.1   19.9 / 19.5 / 17.5
+// The first kernel goes general where this form of it loses (K up to 1280 at 256 rows, 2.9 M weights at 144); between
+// 193 and 256 rows the line at 10 M weights also leaves it general where this form would be up to 2.6 us faster (K of
+// 1536 and 2048 with fewer weights).  The second one (a plain store) takes this form for a short k range per CTA too: up
+// to 3000 rows of operands, 6 blocks x 384 at 1024 x 2816.
 bool stream_gemm_pays(int T, int F, int K, EpiKind kind) {
   const long long weights = static_cast<long long>(F) * K;
   if (T <= 128 || (T <= 192 && weights >= 4000000) || (T <= kMaxT && weights >= 10000000)) return true;
