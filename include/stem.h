@@ -29,7 +29,8 @@
  *     clamped into range so no access leaves the table.  Nothing traps, prints from the
  *     device or throws; there is no CPU fallback.
  *   - dtype 0: fp32 storage, fp32 products and sums (on the tensor cores, three bf16 parts
- *     per operand).  dtype 1: bf16 storage, bf16
+ *     per operand; a contraction with an operand that holds a value of 2^24 or more, an infinity or a
+ *     NaN runs as FMA chains, several times slower).  dtype 1: bf16 storage, bf16
  *     tensor-core products accumulated in fp32, elementwise math in fp32, results
  *     rounded to bf16 (round to nearest even) when stored.
  *   - Shape limits: T <= 2^22; d_model and d_ff multiples of 8 (bf16) or 4 (fp32);
