@@ -36,16 +36,21 @@
 // the weight gradients 126); at 256 positions, 256, 688: 238, 72 and 72 us.  Error against 64 bits:
 // 0.2 - 0.5 of the FMA kernel's for K >= 128, alike at K = 8.
 //
-// A tile is 128 * CTAS rows x BN columns.  CTAS = 2: a pair of CTAs shares each MMA (cta_group::2), each
-// staging its 128 rows of A and half of the columns of B.  Roles per CTA: warp 0 one thread loads with
+// A tile is 128 * CTAS rows x BN columns (64 for a CTA, 128 or, plain stores only, 256 for a pair).  CTAS = 2: a pair of
+// CTAs shares each MMA (cta_group::2), each staging its 128 rows of A and half of the columns of B.  Roles per CTA: warp 0 one thread loads with
 // TMA (one copy brings the three parts of a block), warp 1 allocates tensor memory and (first CTA of a
-// pair) issues the 24 MMAs of a block, warps 2..9 add each finished block sum to their registers (one
-// row per thread, two warps per TMEM lane quarter, each half of the columns) and run the epilogue.
+// pair) issues the 24 MMAs of a block, warps 2..9 (2..17 for 256 columns) add each finished block sum to their registers
+// (one row and 64 columns per thread; 32 for a CTA) and run the epilogue.
 //
 // Bound: a 64-wide block of a pair's tile takes 2100 - 2300 cycles (down at 22 to 176 blocks: 36 to 212 us at 1.965 GHz) for
 // 1536 of MMA.  Each CTA's shared memory is written 72 KB for it and read 6 KB by each of the 24 MMAs (128 rows of
 // A, 64 columns of B): 216 KB, 1730 cycles at 128 bytes a clock, so its bandwidth comes before the MMA rate; what the
 // other 400 - 600 cycles wait for is not known.
+// 256 x 256 tiles of a pair (1.33 times the shared-memory bytes for twice the products, two stages of 96 KB, sixteen adding
+// warps of 64 columns) go where they leave fewer idle pairs or a deeper cut along k: down and dx at 2048 x 1024 x 2816
+// 62.4, 61.5 -> 59.4, 57.4 us (32 clusters of two pairs for 64 pairs' tiles), at 1531 rows 61.5 -> 57.4 and 55.4; the
+// weight gradients at 2048 x 512 x 1500 51.2 -> 47.2.  While they run, 64 of the 74 pairs work at the rate that a
+// large cuBLAS bf16 product reaches in a burst.
 //
 // A launch that would leave SMs idle is cut along k over the CTAs (pairs) of a cluster: each leaves its
 // sums in its own shared memory, and each then adds one share of the columns over the cluster in
@@ -60,23 +65,25 @@ namespace {
 
 constexpr int BM = 128;
 constexpr int BK = 64;
-constexpr int kAccWarps = 8;
-constexpr int kAccThreads = 32 * kAccWarps;
-constexpr int kThreads = 64 + kAccThreads;
+constexpr int kFmaThreads = 256;
 constexpr long long kWaitLimitCycles = 2000000000ll;  // ~1 s at boost clock
 
 template <int BN, int CTAS>
 struct Smem {
-  static constexpr int kStages = 3;
+  static constexpr bool kWide = BN == 256;           // 256 x 256 tiles of a CTA pair
+  static constexpr int kAccWarps = kWide ? 16 : 8;
+  static constexpr int kAccThreads = 32 * kAccWarps;
+  static constexpr int kThreads = 64 + kAccThreads;
+  static constexpr int kStages = kWide ? 2 : 3;
   static constexpr int kBCols = BN / CTAS;           // columns of B staged by one CTA
-  static_assert(kBCols == 64, "B is one 64-wide swizzled block per part");
+  static_assert(kBCols % 64 == 0, "B is 64-wide swizzled blocks");
   static constexpr int kAPart = BM * BK * 2;
   static constexpr int kBPart = kBCols * BK * 2;
   static constexpr int kStageBytes = 3 * (kAPart + kBPart);
   static constexpr int kBarOffset = kStages * kStageBytes;
   // Block sums in flight in tensor memory: the epilogue of a tile holds the accumulating warps up for
   // several blocks' time, during which the MMAs go on with the next tile.
-  static constexpr int kBufs = 4;
+  static constexpr int kBufs = kWide ? 2 : 4;
   static constexpr int kNumBars = 2 * kStages + 2 * kBufs + 1;   // full, empty, tmem_full, tmem_empty, drain
   static constexpr int kTotal = kBarOffset + kNumBars * 8 + 16 + 1024;  // + alignment slack
   static_assert(kTotal <= 232448, "exceeds the shared memory a CTA can have");
@@ -252,10 +259,11 @@ __device__ __forceinline__ int table_row(const EpiParams& ep, int m) {
 }
 
 // ---- operands that the parts cannot carry --------------------------------------------------------
+template <int THREADS>
 __device__ __forceinline__ bool any_word(const uint32_t* words, int n, int et) {
   uint32_t any = 0;
 #pragma unroll 4
-  for (int i = et; i < n; i += kAccThreads) any |= words[i];
+  for (int i = et; i < n; i += THREADS) any |= words[i];
   return any != 0;
 }
 // The outputs of the whole launch by the accumulating warps of its CTAs, 64 x 64 at a time: one chain of FMAs
@@ -278,7 +286,7 @@ __device__ __noinline__ void fma_tiles(const EpiParams& ep, const Product& p1, c
     auto fetch = [&](int k0) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int idx = et + i * kAccThreads;
+        const int idx = et + i * kFmaThreads;
         const int am = A_MN ? idx % FT : idx / FK, ak = k0 + (A_MN ? idx / FT : idx % FK);
         const int bn = B_MN ? idx % FT : idx / FK, bk = k0 + (B_MN ? idx / FT : idx % FK);
         ra[i] = m0 + am < pr.M && ak < K
@@ -293,11 +301,11 @@ __device__ __noinline__ void fma_tiles(const EpiParams& ep, const Product& p1, c
       float* Bs = As + FK * kPitch;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int idx = et + i * kAccThreads;
+        const int idx = et + i * kFmaThreads;
         As[(A_MN ? idx / FT : idx % FK) * kPitch + (A_MN ? idx % FT : idx / FK)] = ra[i];
         Bs[(B_MN ? idx / FT : idx % FK) * kPitch + (B_MN ? idx % FT : idx / FK)] = rb[i];
       }
-      ptx::named_sync(1, kAccThreads);      // (nobody still reads the other buffer's last step behind this one)
+      ptx::named_sync(2, kFmaThreads);      // (nobody still reads the other buffer's last step behind this one)
       if (k0 + FK < K) fetch(k0 + FK);
 #pragma unroll
       for (int kk = 0; kk < FK; ++kk) {
@@ -326,13 +334,14 @@ __device__ __noinline__ void fma_tiles(const EpiParams& ep, const Product& p1, c
 struct Maps { CUtensorMap A, B, A2, B2; };   // [3][rows, cols] parts; the second product's
 
 template <bool A_MN, bool B_MN, int KIND, int BN, int CTAS>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(Smem<BN, CTAS>::kThreads, 1)
 split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Product p1,
                   const __grid_constant__ Product p2, int K, int ksplit, const __grid_constant__ EpiParams ep) {
   using L = Smem<BN, CTAS>;
   constexpr int STAGES = L::kStages;
   constexpr int TM = BM * CTAS;
   constexpr int BUFS = L::kBufs;
+  constexpr int kAccWarps = L::kAccWarps, kAccThreads = L::kAccThreads;
   constexpr uint32_t kTmemCols = BUFS * BN;
   static_assert(kTmemCols <= 512, "tensor memory has 512 columns");
   extern __shared__ uint8_t smem_raw[];
@@ -415,14 +424,19 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
             if (CTAS == 2) ptx::tma_load_3d_pair(dst, map, fb, c0, c1, 0); else ptx::tma_load_3d(dst, map, fb, c0, c1, 0);
           };
           const int k0 = kb * BK;
-          // K-major: [part][128 rows][64 k].  MN-major: two 64-wide blocks, each [part][64 k][64 m].
+          // K-major: [part][rows][64 k].  MN-major: 64-wide blocks, each [part][64 k][64 m or n].
           if (A_MN) {
             load(a_dst, mapA, m0, k0);
             load(a_dst + 3 * L::kAPart / 2, mapA, m0 + 64, k0);
           } else {
             load(a_dst, mapA, k0, m0);
           }
-          if (B_MN) load(b_dst, mapB, n0, k0); else load(b_dst, mapB, k0, n0);
+          if (B_MN) {
+#pragma unroll
+            for (int j = 0; j < L::kBCols / 64; ++j) load(b_dst + j * (3 * 64 * BK * 2), mapB, n0 + 64 * j, k0);
+          } else {
+            load(b_dst, mapB, k0, n0);
+          }
           ++issued;
           if (++s == STAGES) { s = 0; ph ^= 1u; }
         }
@@ -448,14 +462,15 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
           constexpr int ia[kTerms] = {2, 0, 1, 1, 0, 0}, ib[kTerms] = {0, 2, 1, 0, 1, 0};   // smallest terms first
           // bytes from one part of A to the next, and (MN-major) from one 64-wide block to the next
           constexpr int a_part = A_MN ? L::kAPart / 2 : L::kAPart, a_block = 3 * L::kAPart / 2;
+          constexpr int b_part = B_MN ? 64 * BK * 2 : L::kBPart, b_block = 3 * 64 * BK * 2;
 #pragma unroll
           for (int term = 0; term < kTerms; ++term) {
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk) {
-              const uint32_t a = a_src + ia[term] * a_part, b = b_src + ib[term] * L::kBPart;
+              const uint32_t a = a_src + ia[term] * a_part, b = b_src + ib[term] * b_part;
               const uint64_t ad = A_MN ? ptx::make_smem_desc(a + kk * (16 * 128), a_block, 1024)
                                        : ptx::make_smem_desc(a + kk * 32, 16, 1024);
-              const uint64_t bd = B_MN ? ptx::make_smem_desc(b + kk * (16 * 128), L::kBPart, 1024)
+              const uint64_t bd = B_MN ? ptx::make_smem_desc(b + kk * (16 * 128), b_block, 1024)
                                        : ptx::make_smem_desc(b + kk * 32, 16, 1024);
               if (CTAS == 2) ptx::mma_bf16_ss_pair(d_tmem, ad, bd, idesc, (term > 0 || kk > 0) ? 1u : 0u);
               else ptx::mma_bf16_ss(d_tmem, ad, bd, idesc, (term > 0 || kk > 0) ? 1u : 0u);
@@ -475,23 +490,24 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
       }
     }
   } else {
-    constexpr int kCols = BN / 2;           // columns per thread
+    constexpr int kCols = 4 * BN / kAccWarps;   // columns per thread
+    constexpr int kLd = L::kWide ? 16 : 32;     // columns read from tensor memory at once (eighteen warps: 96 registers)
     const int q = warp & 3;                 // TMEM lane quarter this warp may read
-    const int half = (warp - 2) >> 2;       // which half of the tile's columns it handles
+    const int group = (warp - 2) >> 2;      // which kCols of the tile's columns it handles
     const int r = q * 32 + lane;            // row among this CTA's 128
     int buf = 0; uint32_t bph = 0;
     float acc[kCols], e[8], g[8];
     const int share = kCols / ksplit;       // columns of a tile that this thread finishes
     const int et = threadIdx.x - 64;
-    bool beyond = any_word(p1.a_words, p1.a_n, et) || any_word(p1.b_words, p1.b_n, et);
-    if (KIND == kEpiStore && tiles2 > 0) beyond = beyond || any_word(p2.a_words, p2.a_n, et) || any_word(p2.b_words, p2.b_n, et);
+    bool beyond = any_word<kAccThreads>(p1.a_words, p1.a_n, et) || any_word<kAccThreads>(p1.b_words, p1.b_n, et);
+    if (KIND == kEpiStore && tiles2 > 0) beyond = beyond || any_word<kAccThreads>(p2.a_words, p2.a_n, et) || any_word<kAccThreads>(p2.b_words, p2.b_n, et);
     beyond = ptx::named_sync_or(1, kAccThreads, beyond);
     int id = 0;
     for (int tile = tile0; ok && tile < num_tiles; tile += tile_step) {
       const bool second = KIND == kEpiStore && tile >= tiles1;
       const Product& pr = second ? p2 : p1;
       const int tt = second ? tile - tiles1 : tile, tm = second ? tiles_m2 : tiles_m1;
-      const int m = tt % tm * TM + rank * BM + r, n0 = tt / tm * BN + half * kCols;
+      const int m = tt % tm * TM + rank * BM + r, n0 = tt / tm * BN + group * kCols;
 #pragma unroll
       for (int c = 0; c < kCols; ++c) acc[c] = 0.0f;
       // the epilogue's first operands are on their way while the blocks are summed
@@ -506,13 +522,13 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
           ok = false; break;
         }
         ptx::tc_fence_after();
-        const uint32_t t_row = tmem_base + buf * BN + half * kCols + (static_cast<uint32_t>(q * 32) << 16);
+        const uint32_t t_row = tmem_base + buf * BN + group * kCols + (static_cast<uint32_t>(q * 32) << 16);
 #pragma unroll
-        for (int c = 0; c < kCols; c += 32) {
-          uint32_t v[32];
-          ptx::tmem_ld_32x32(t_row + c, v);
+        for (int c = 0; c < kCols; c += kLd) {
+          uint32_t v[kLd];
+          if constexpr (kLd == 32) ptx::tmem_ld_32x32(t_row + c, v); else ptx::tmem_ld_32x16(t_row + c, v);
           ptx::tmem_ld_wait();
-          if (c + 32 == kCols) {   // read out: the buffer goes back to the MMA issuer
+          if (c + kLd == kCols) {   // read out: the buffer goes back to the MMA issuer
             ptx::tc_fence_before();
             __syncwarp();
             if (lane == 0) {
@@ -521,7 +537,7 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
             }
           }
 #pragma unroll
-          for (int i = 0; i < 32; ++i) acc[c + i] += __uint_as_float(v[i]);
+          for (int i = 0; i < kLd; ++i) acc[c + i] += __uint_as_float(v[i]);
         }
         if (++buf == BUFS) { buf = 0; bph ^= 1u; }
       }
@@ -544,7 +560,7 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
       } else {
         // This CTA's copies have landed and its MMAs (a pair's: of both) are complete, so the operand
         // ring is free: leave the sums there, column by column (128 rows of a column side by side).
-        float* part = reinterpret_cast<float*>(base_ptr) + static_cast<size_t>(half) * kCols * BM + r;
+        float* part = reinterpret_cast<float*>(base_ptr) + static_cast<size_t>(group) * kCols * BM + r;
 #pragma unroll
         for (int c = 0; c < kCols; ++c) part[c * BM] = acc[c];
       }
@@ -556,9 +572,9 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
       const bool second = KIND == kEpiStore && tile0 >= tiles1;
       const Product& pr = second ? p2 : p1;
       const int tt = second ? tile0 - tiles1 : tile0, tm = second ? tiles_m2 : tiles_m1;
-      const int m = tt % tm * TM + rank * BM + r, n0 = tt / tm * BN + half * kCols + slice * share;
+      const int m = tt % tm * TM + rank * BM + r, n0 = tt / tm * BN + group * kCols + slice * share;
       if (ok && m < pr.M && !beyond) {
-        const uint32_t mine = base + 4u * (static_cast<uint32_t>(half * kCols + slice * share) * BM + r);
+        const uint32_t mine = base + 4u * (static_cast<uint32_t>(group * kCols + slice * share) * BM + r);
         const int end = min(n0 + share, pr.N);
 #pragma unroll 1
         for (int n = n0; n < end; n += 8) {
@@ -583,7 +599,7 @@ split_gemm_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Pro
       __syncwarp();
     }
     // Every copy into this CTA's ring and every MMA on it is complete (as above), and no CTA of the cluster reads it.
-    if (beyond && !ptx::named_sync_or(1, kAccThreads, !ok))
+    if (beyond && !ptx::named_sync_or(1, kAccThreads, !ok) && et < kFmaThreads)
       fma_tiles<A_MN, B_MN, KIND>(ep, p1, p2, K, reinterpret_cast<float*>(base_ptr), et);
     __syncwarp();
   }
@@ -631,32 +647,35 @@ bool encode_parts(CUtensorMap* map, const Parts& p, int box_rows) {
 // Tile shape and k split.  The time of a launch is its rounds of tiles over the SMs times the k blocks of
 // a tile times a block's cost (1750 cycles for either shape, by shared-memory bytes: a pair's
 // measured 2100 - 2300, but the plan only compares; a pair's tile is four times as large on twice the SMs), plus a tile's own latencies, plus what adding the slices
-// costs.  A cluster has at most 8 CTAs, and a slice at least 2 blocks.
-struct Plan { bool pair; int ksplit; };
+// costs.  A cluster has at most 8 CTAs, and a slice at least 2 blocks.  A block of a 256 x 256 tile counts as 1.5 of
+// the others; a tie goes to the narrower tile: at 1.31 the weight gradients of 2048 x 1024 x 2816 (3 rounds of 176 tiles or 2
+// of 88) went from 125 to 139 us, those of 600 rows from 49 to 57.
+struct Plan { int ctas, bn, ksplit; };
 long long tile_count(int M, int N, int tm, int bn) { return static_cast<long long>((M + tm - 1) / tm) * ((N + bn - 1) / bn); }
-Plan make_plan(int M1, int N1, int M2, int N2, int K, bool pairs) {
+Plan make_plan(int M1, int N1, int M2, int N2, int K, bool pairs, bool wide) {
+  struct Shape { int ctas, bn; double block; };
+  constexpr Shape shapes[3] = {{2, 128, 1750.0}, {1, 64, 1750.0}, {2, 256, 2625.0}};
   const int k_blocks = (K + BK - 1) / BK;
-  Plan best{pairs, 1};
+  Plan best{1, 64, 1};
   double best_cost = 0.0;
-  for (bool pair : {true, false}) {
-    if (pair && !pairs) continue;
-    const int ctas = pair ? 2 : 1, slots = device_sm_count() / ctas;
-    const long long tiles = tile_count(M1, N1, BM * ctas, 64 * ctas) + tile_count(M2, N2, BM * ctas, 64 * ctas);
-    for (int sp = 1; sp * ctas <= 8; sp *= 2) {
+  for (const Shape& s : shapes) {
+    if ((s.ctas == 2 && !pairs) || (s.bn == 256 && !wide)) continue;
+    const int slots = device_sm_count() / s.ctas;
+    const long long tiles = tile_count(M1, N1, BM * s.ctas, s.bn) + tile_count(M2, N2, BM * s.ctas, s.bn);
+    for (int sp = 1; sp * s.ctas <= 8; sp *= 2) {
       if (sp > 1 && (tiles * sp > slots || k_blocks < 2 * sp)) break;
-      const int at_once = clusters_at_once(ctas * sp);
+      const int at_once = clusters_at_once(s.ctas * sp);
       const double rounds = static_cast<double>((tiles + at_once - 1) / at_once);
-      const double cost = rounds * ((k_blocks + sp - 1) / sp * 1750.0) + 3000.0 + (sp > 1 ? 2500.0 : 0.0);
-      if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = {pair, sp}; }
+      const double cost = rounds * ((k_blocks + sp - 1) / sp * s.block) + 3000.0 + (sp > 1 ? 2500.0 : 0.0);
+      if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = {s.ctas, s.bn, sp}; }
     }
   }
   return best;
 }
 
-template <bool A_MN, bool B_MN, int KIND, int CTAS>
+template <bool A_MN, bool B_MN, int KIND, int CTAS, int BN = 64 * CTAS>
 cudaError_t launch_inst(const SplitProduct& a, const SplitProduct& b, int K, int ksplit, const EpiParams& ep,
                         cudaStream_t stream) {
-  constexpr int BN = 64 * CTAS;
   using L = Smem<BN, CTAS>;
   auto kern = split_gemm_kernel<A_MN, B_MN, KIND, BN, CTAS>;
   static PerDeviceOnce configured;
@@ -665,7 +684,7 @@ cudaError_t launch_inst(const SplitProduct& a, const SplitProduct& b, int K, int
       }))
     return ce;
   Maps maps;
-  const int rows_a = A_MN ? BK : BM, rows_b = 64;
+  const int rows_a = A_MN ? BK : BM, rows_b = B_MN ? BK : L::kBCols;
   bool good = encode_parts(&maps.A, a.A3, rows_a) && encode_parts(&maps.B, a.B3, rows_b);
   if (b.M > 0) good = good && encode_parts(&maps.A2, b.A3, rows_a) && encode_parts(&maps.B2, b.B3, rows_b);
   else { maps.A2 = maps.A; maps.B2 = maps.B; }
@@ -685,7 +704,7 @@ cudaError_t launch_inst(const SplitProduct& a, const SplitProduct& b, int K, int
   const long long units = ksplit > 1 ? tiles * ksplit : (tiles < slots ? tiles : slots);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(units * CTAS));
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3(L::kThreads);
   cfg.dynamicSmemBytes = L::kTotal;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -705,8 +724,11 @@ cudaError_t launch_inst(const SplitProduct& a, const SplitProduct& b, int K, int
 template <bool A_MN, bool B_MN, int KIND>
 cudaError_t launch_planned(const SplitProduct& a, const SplitProduct& b, int K, const EpiParams& ep, bool pairs,
                            cudaStream_t stream) {
-  const Plan pl = make_plan(a.M, a.N, b.M, b.N, K, pairs);
-  if (pl.pair) return launch_inst<A_MN, B_MN, KIND, 2>(a, b, K, pl.ksplit, ep, stream);
+  const Plan pl = make_plan(a.M, a.N, b.M, b.N, K, pairs, KIND == kEpiStore);
+  if constexpr (KIND == kEpiStore) {
+    if (pl.bn == 256) return launch_inst<A_MN, B_MN, KIND, 2, 256>(a, b, K, pl.ksplit, ep, stream);
+  }
+  if (pl.ctas == 2) return launch_inst<A_MN, B_MN, KIND, 2>(a, b, K, pl.ksplit, ep, stream);
   return launch_inst<A_MN, B_MN, KIND, 1>(a, b, K, pl.ksplit, ep, stream);
 }
 

@@ -68,3 +68,30 @@ def test_inputs_the_parts_cannot_carry():
         if m.any():
             scale = b[r][m].abs().max()
             assert (a[r][m] - b[r][m]).abs().max() <= 4e-6 * scale, r      # sqrt(d) 2^-24 each, doubled
+
+
+# Tiles of 256 x 256: cut along k and not, one round and two, in every layout of a plain store; ragged in both extents
+@pytest.mark.parametrize("T,d,F", [(1801, 700, 1200), (2500, 1000, 260), (2500, 260, 1000)])
+def test_layer_fp32_wide_tiles(T, d, F):
+    w = synth.Workload("t", T, d, F, 500, "fp32", "zipf")
+    _full_parity(w, synth.make_inputs(w, seed=34), B.DTYPE_FP32, TOL_FP32)
+
+
+def test_wide_tiles_that_the_parts_cannot_carry():
+    """An infinity sends the launch to FMA chains: finite where the FMA kernels are, and as close to them as two fp32 sums."""
+    T, d, F, V = 1801, 700, 1200, 50
+    out = []
+    for flags in (0, B.FLAG_SIMT):
+        w = synth.Workload("t", T, d, F, V, "fp32", "zipf")
+        st = runner.state_from_numpy(synth.make_inputs(w, seed=35), B.DTYPE_FP32, V, flags=flags, backward=False)
+        st.W_down[17, 9] = float("inf")
+        st.dedup()
+        st.forward()
+        assert st.status() == B.OK
+        out.append(st.bufs["y"].double())
+    a, b = out
+    assert torch.equal(a.isfinite(), b.isfinite())
+    fin = a.isfinite()
+    assert fin.any() and not fin.all()
+    # both are chains of K <= 1200 fp32 additions of an H that differs by a few 2^-24 of its row
+    assert (a[fin] - b[fin]).norm() <= TOL_FP32 * b[fin].norm()
